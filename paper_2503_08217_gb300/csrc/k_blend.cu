@@ -19,8 +19,8 @@
 // transmittance before each splat is recovered from the stored final value as
 // T <- T / (1 - alpha), so no per-pixel lists are kept; a lane's two pixels
 // of a column again form one packed pair. Per splat the nine
-// adjoints (uv, conic, opacity, rgb) are summed over the warp with shuffles,
-// then over the CTA in shared memory (one shared atomic per splat and warp),
+// adjoints (uv, conic, opacity, rgb) are summed over the warp through shared
+// memory, then over the CTA (one shared atomic per two splats and warp),
 // and flushed to global memory with one vector atomic per four floats.
 #include "s3r_internal.cuh"
 
@@ -34,7 +34,7 @@ namespace {
 #define S3R_BLEND_FWD_BATCH 64    // splats staged per batch (forward)
 #endif
 #ifndef S3R_BLEND_FWD_BLOCKS
-#define S3R_BLEND_FWD_BLOCKS 20   // resident forward blocks per SM (register budget)
+#define S3R_BLEND_FWD_BLOCKS 18   // resident forward blocks per SM (register budget)
 #endif
 #ifndef S3R_BLEND_BWD_BATCH
 #define S3R_BLEND_BWD_BATCH 64    // splats staged per batch (backward)
@@ -408,6 +408,28 @@ __device__ __forceinline__ bool box_misses(const float4 b, const Band& t) {
 // arithmetic is the exponent and alpha of stage_splat's comment, in that
 // order, so the backward's recomputation takes the same decisions.
 constexpr int kBatchFwd = S3R_BLEND_FWD_BATCH;
+// The forward's decision for one pixel as one predicate chain (three compares,
+// three selects; written as compiler booleans the same decisions took about
+// twice the integer-pipe instructions, and that pipe is the forward's busiest).
+// `floor_` is the least alpha the pixel still takes: 1/255 until it stops, then
+// infinity. The splat is taken where p <= 0, alpha >= floor_ and the
+// transmittance nT it would leave is not under 1e-4; where only the last fails
+// the pixel stops. It took 6.5 % off the kernel's instructions. Returns the applied alpha and moves the last position.
+__device__ __forceinline__ float blend_alpha(float p, float al, float nT, int pos, float& floor_,
+                                             int& last) {
+  float ab;
+  asm("{\n\t.reg .pred q, s, b;\n\t"
+      "setp.leu.f32 q, %3, 0f00000000;\n\t"
+      "setp.geu.and.f32 q, %4, %1, q;\n\t"
+      "setp.lt.and.f32 s|b, %5, %7, q;\n\t"
+      "selp.f32 %0, %4, 0f00000000, b;\n\t"
+      "selp.b32 %2, %6, %2, b;\n\t"
+      "selp.f32 %1, 0f7F800000, %1, s;\n\t}"
+      : "=&f"(ab), "+f"(floor_), "+r"(last)
+      : "f"(p), "f"(al), "f"(nT), "r"(pos), "f"(kTStop));
+  return ab;
+}
+
 // One splat of the forward's walk over a warp's four pixels per lane (two
 // packed pairs). kClamp: the splat's opacity exceeds 0.99, so alpha = o G may
 // reach the 0.99 cap; for o <= 0.99 it cannot (G = 2^p <= 1 where p <= 0, up
@@ -419,11 +441,11 @@ __device__ __forceinline__ void fwd_splat(const float4 q0, const float4 q1, cons
                                           const float4 q3, const float2 qu, const f2 FY,
                                           const f2 (&FX)[2], const f2 ONE, int pos, f2 (&T2)[2],
                                           f2 (&C2)[2][3], int (&last)[kBandPix],
-                                          int (&endp)[kBandPix], bool (&done)[kBandPix],
+                                          int (&endp)[kBandPix], float (&floor_)[kBandPix],
                                           uint32_t& n_eval, bool& any_blend) {
   // a blended pixel takes alpha >= 1/255 > 0, a skipped one 0: the splat was
   // blended somewhere in the lane's pixels iff the applied alphas sum above 0
-  f2 ab_sum = pk(0.f, 0.f);
+  f2 ab_sum;
   const f2 A2 = pk(q0.x, q0.y), B2 = pk(q0.z, q0.w), C2c = pk(q1.x, q1.y), O2 = pk(q1.z, q1.w);
   const f2 R2 = pk(q2.x, q2.y), G2 = pk(q2.z, q2.w), Bl2 = pk(q3.x, q3.y), V2 = pk(q3.z, q3.w);
   const f2 U2 = pk(qu.x, qu.y);
@@ -435,36 +457,25 @@ __device__ __forceinline__ void fwd_splat(const float4 q0, const float4 q1, cons
   for (int c = 0; c < 2; ++c) {
     const f2 dx = sub2(U2, FX[c]);
     const f2 pw = fma2(dx, fma2(A2, dx, bdy), cdy);
-    float p[2], G[2];
+    float p[2], raw[2];
     upk(pw, p[0], p[1]);
-    G[0] = ex2_approx(p[0]);
-    G[1] = ex2_approx(p[1]);
-    float raw[2];
-    upk(mul2(O2, pk(G[0], G[1])), raw[0], raw[1]);
+    upk(mul2(O2, pk(ex2_approx(p[0]), ex2_approx(p[1]))), raw[0], raw[1]);
     float al[2], ab[2];
-    bool blend[2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int k = c * kBandRows + r;
-      al[r] = kClamp ? fminf(kAlphaMax, raw[r]) : raw[r];
-      if constexpr (kCount) n_eval += done[k] ? 0u : 1u;
-      blend[r] = !done[k] && !(p[r] > 0.f) && !(al[r] < kAlphaMin);
-    }
+    for (int r = 0; r < 2; ++r) al[r] = kClamp ? fminf(kAlphaMax, raw[r]) : raw[r];
     float nT[2];
     upk(mul2(T2[c], sub2(ONE, pk(al[0], al[1]))), nT[0], nT[1]);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int k = c * kBandRows + r;
-      const bool stop = blend[r] && (nT[r] < kTStop);
-      blend[r] = blend[r] && !stop;
+      const bool was_done = floor_[k] > 1.f;
+      if constexpr (kCount) n_eval += was_done ? 0u : 1u;
       // one select: T (1 - 0) = T exactly where the splat is not blended
-      ab[r] = blend[r] ? al[r] : 0.f;
-      last[k] = blend[r] ? pos : last[k];
-      if constexpr (kCount) endp[k] = stop ? pos : endp[k];
-      done[k] = done[k] || stop;
+      ab[r] = blend_alpha(p[r], al[r], nT[r], pos, floor_[k], last[k]);
+      if constexpr (kCount) endp[k] = !was_done && floor_[k] > 1.f ? pos : endp[k];
     }
     const f2 AB = pk(ab[0], ab[1]);
-    ab_sum = add2(ab_sum, AB);
+    ab_sum = c == 0 ? AB : add2(ab_sum, AB);
     const f2 w = mul2(AB, T2[c]);
     C2[c][0] = fma2(R2, w, C2[c][0]);
     C2[c][1] = fma2(G2, w, C2[c][1]);
@@ -476,8 +487,15 @@ __device__ __forceinline__ void fwd_splat(const float4 q0, const float4 q1, cons
   any_blend = s0 + s1 > 0.f;
 }
 
-// S3R_BLEND_FWD_BLOCKS: 20 blocks per SM (48 registers, a small spill)
-// measured fastest: 16 (64 registers) 6 % slower, 22 and 24 11 % slower.
+__device__ __forceinline__ bool all_stopped(const float (&floor_)[kBandPix]) {
+  static_assert(kBandPix == 4, "four pixels per lane");
+  return fminf(fminf(floor_[0], floor_[1]), fminf(floor_[2], floor_[3])) > 1.f;
+}
+
+// S3R_BLEND_FWD_BLOCKS: 18 blocks per SM (56 registers). At the surround rig
+// (27.7M pairs, 1.07G evaluated) 18 blocks took 1.043 ms, 20 (48 registers)
+// 1.084 ms and 16 (64 registers) 1.148 ms: the kernel needs the warps, and a
+// few registers more than 48 end the spills.
 template <bool kCount>
 __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fwd(const __grid_constant__ ViewSet vs,
                                                             BlendArgs a) {
@@ -515,9 +533,8 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
     // per column c: the pair (row 0, row 1); scalar per-pixel state k = 2c + r
     f2 T2[2], C2[2][3];
     int last[kBandPix], endp[kBandPix];
-    bool done[kBandPix];
+    float floor_[kBandPix];   // least alpha taken; infinity once the pixel has stopped
     uint32_t n_eval = 0;
-    bool all_done = true;
   #pragma unroll
     for (int c = 0; c < 2; ++c) {
       T2[c] = ONE;
@@ -526,17 +543,15 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
       for (int r = 0; r < kBandRows; ++r) {
         const int k = c * kBandRows + r;
         last[k] = 0;
-        done[k] = !(P.X0 + 8 * c < vi.width && P.Y0 + 4 * r < vi.height);
-        endp[k] = done[k] ? 0 : n;      // positions walked
-        all_done = all_done && done[k];
+        const bool inside = P.X0 + 8 * c < vi.width && P.Y0 + 4 * r < vi.height;
+        floor_[k] = inside ? kAlphaMin : INFINITY;
+        endp[k] = inside ? n : 0;      // positions walked
       }
     }
     uint32_t* wbits = a.contrib + warp * a.contrib_words;
     for (int b0 = 0; b0 < n; b0 += kBatchFwd) {
-      // the pixels' done flags are folded once per chunk and batch, not per splat
-  #pragma unroll
-      for (int k = 0; k < kBandPix; ++k) all_done = all_done && done[k];
-      if (__syncthreads_count(all_done) == kBandThreads) break;
+      // whether every pixel has stopped: tested once per chunk and batch, not per splat
+      if (__syncthreads_and(all_stopped(floor_))) break;
       for (int i = threadIdx.x; i < kBatchFwd && b0 + i < n; i += kBandThreads) {
         const uint32_t s = a.sorted_splats[range.x + b0 + i];
         const uint4 t0 = a.sp_tin[2 * (size_t)s], t1 = a.sp_tin[2 * (size_t)s + 1];
@@ -557,10 +572,7 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
       __syncthreads();
       const int m = min(kBatchFwd, n - b0);
       for (int c0 = 0; c0 < m; c0 += 32) {
-        all_done = true;
-  #pragma unroll
-        for (int k = 0; k < kBandPix; ++k) all_done = all_done && done[k];
-        if (__all_sync(0xffffffffu, all_done)) break;
+        if (__all_sync(0xffffffffu, all_stopped(floor_))) break;
         // which of the next 32 splats can reach alpha >= 1/255 in this warp's band
         const int jl = c0 + (int)lane;
         bool reach = false;
@@ -581,10 +593,10 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
           bool any_blend = false;
           // warp-uniform: every lane walks the same splat
           if (q1.z > kAlphaMax)
-            fwd_splat<kCount, true>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, done,
+            fwd_splat<kCount, true>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, floor_,
                                     n_eval, any_blend);
           else
-            fwd_splat<kCount, false>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, done,
+            fwd_splat<kCount, false>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, floor_,
                                      n_eval, any_blend);
           if (__any_sync(0xffffffffu, any_blend)) blended |= 1u << (j - c0);
         }
@@ -645,31 +657,19 @@ __device__ __forceinline__ float select_f(bool a, float x, float y) {
   return r;
 }
 
-// Sum eight values over the warp with 9 shuffles instead of 8 x 5: at each
-// butterfly level every lane keeps half of its remaining values and sends the
-// other half to its partner. On return, lane l holds the warp total of value
-// index 4*bit4(l) + 2*bit3(l) + bit2(l); lanes 4m (m = 0..7) hold value m.
-__device__ __forceinline__ float warp_sum8_transposed(const float v[8], uint32_t lane) {
-  const bool b4 = lane & 16u, b3 = lane & 8u, b2 = lane & 4u;
-  float k4[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float send = select_f(b4, v[j], v[j + 4]);
-    const float keep = select_f(b4, v[j + 4], v[j]);
-    k4[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-  float k2[2];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float send = select_f(b3, k4[j], k4[j + 2]);
-    const float keep = select_f(b3, k4[j + 2], k4[j]);
-    k2[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  const float send = select_f(b2, k2[0], k2[1]);
-  float k1 = select_f(b2, k2[1], k2[0]) + __shfl_xor_sync(0xffffffffu, send, 4);
-  k1 += __shfl_xor_sync(0xffffffffu, k1, 2);
-  k1 += __shfl_xor_sync(0xffffffffu, k1, 1);
-  return k1;
+// The backward's decision for one pixel as one predicate chain: the splat's
+// alpha where the forward blended it (position before the pixel's last
+// contributor, p <= 0, alpha >= 1/255), else 0.
+__device__ __forceinline__ float taken_alpha(float p, float al, int pos, int last) {
+  float r;
+  asm("{\n\t.reg .pred q;\n\t"
+      "setp.lt.s32 q, %3, %4;\n\t"
+      "setp.leu.and.f32 q, %1, 0f00000000, q;\n\t"
+      "setp.geu.and.f32 q, %2, %5, q;\n\t"
+      "selp.f32 %0, %2, 0f00000000, q;\n\t}"
+      : "=f"(r)
+      : "f"(p), "f"(al), "r"(pos), "r"(last), "f"(kAlphaMin));
+  return r;
 }
 
 __device__ __forceinline__ void red_shared(float* addr, float v) {
@@ -721,16 +721,21 @@ __device__ __forceinline__ void bwd_init(BwdPixel& q, const BlendArgs& a, const 
 }
 
 // One splat of the backward's walk (see above) over a lane's two packed
-// pixel pairs: updates T and Bd, returns the lane's shares of the nine sums
-// (g0..g3 scalar, g4..g8 as row pairs). kClamp as for fwd_splat, per splat.
+// pixel pairs: updates T and Bd, returns the lane's shares of the nine sums in
+// g. kClamp as for fwd_splat, per splat.
+//
+// A pixel that does not take the splat gets alpha 0: 1 / (1 - 0) is exactly 1,
+// so T, the weight and every sum are left unchanged by the same arithmetic,
+// with one select per pixel. Without the cap, alpha = o G, so G dL/dalpha (the
+// opacity's term) is (alpha dL/dalpha) / o and the sum of the power's adjoint
+// serves both; the division is made once per splat at the flush.
 template <bool kCount, bool kClamp>
 __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, const float4 q2,
                                           const float4 q3, const float2 qu, const f2 FY,
                                           const f2 (&FX)[2], const f2 ONE, int pos,
                                           const int (&last)[kBandPix], f2 (&T2)[2], f2 (&Bd2)[2],
                                           const f2 (&Q0)[2], const f2 (&Q1)[2], const f2 (&Q2)[2],
-                                          uint32_t& n_eval, float (&g)[4], f2& g4, f2& g5, f2& g6,
-                                          f2& g7, f2& g8) {
+                                          uint32_t& n_eval, float (&g)[9]) {
   constexpr int kRows = kBandRows;
   const f2 A2 = pk(q0.x, q0.y), B2 = pk(q0.z, q0.w), C2c = pk(q1.x, q1.y), O2 = pk(q1.z, q1.w);
   const f2 R2 = pk(q2.x, q2.y), G2 = pk(q2.z, q2.w), Bl2 = pk(q3.x, q3.y), V2 = pk(q3.z, q3.w);
@@ -738,70 +743,108 @@ __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, cons
   const f2 dy = sub2(V2, FY);
   const f2 bdy = mul2(B2, dy);
   const f2 cdy = mul2(mul2(C2c, dy), dy);
-  float dyv[2];
-  upk(dy, dyv[0], dyv[1]);
-  g[0] = g[1] = g[2] = g[3] = 0.f;
-  g4 = g5 = g6 = g7 = g8 = pk(0.f, 0.f);
+  f2 pdy_all, w0, w1, w2;
+  float D[2], E[2], dx[2];
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const f2 dx2 = sub2(U2, FX[c]);
     const f2 pw = fma2(dx2, fma2(A2, dx2, bdy), cdy);
-    float p[2], G[2], raw[2], al[2], inv[2];
-    bool act[2], live[2];
+    float p[2], raw[2], al[2], inv[2];
     upk(pw, p[0], p[1]);
-    G[0] = ex2_approx(p[0]);
-    G[1] = ex2_approx(p[1]);
-    upk(mul2(O2, pk(G[0], G[1])), raw[0], raw[1]);
+    upk(mul2(O2, pk(ex2_approx(p[0]), ex2_approx(p[1]))), raw[0], raw[1]);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int k = c * kRows + r;
       al[r] = kClamp ? fminf(kAlphaMax, raw[r]) : raw[r];
       if constexpr (kCount) n_eval += pos < last[k] ? 1u : 0u;
-      act[r] = (pos < last[k]) && !(p[r] > 0.f) && !(al[r] < kAlphaMin);
-      // alpha = 0.99 is constant in o; without the cap alpha = o G throughout
-      live[r] = kClamp ? act[r] && !(raw[r] > kAlphaMax) : act[r];
+      al[r] = taken_alpha(p[r], al[r], pos, last[k]);
     }
     const f2 AL = pk(al[0], al[1]);
     upk(sub2(ONE, AL), inv[0], inv[1]);
     inv[0] = rcp_approx(inv[0]);
     inv[1] = rcp_approx(inv[1]);
-    // T before this splat where it was blended; Bd the colour behind it
-    float Tn[2], Tc[2];
-    upk(mul2(T2[c], pk(inv[0], inv[1])), Tn[0], Tn[1]);
-    upk(T2[c], Tc[0], Tc[1]);
-    Tc[0] = select_f(act[0], Tn[0], Tc[0]);
-    Tc[1] = select_f(act[1], Tn[1], Tc[1]);
-    T2[c] = pk(Tc[0], Tc[1]);
+    // T before this splat; Bd the colour behind it
+    T2[c] = mul2(T2[c], pk(inv[0], inv[1]));
     const f2 cd = fma2(R2, Q0[c], fma2(G2, Q1[c], mul2(Bl2, Q2[c])));
     const f2 dal = fma2(T2[c], cd, mul2(Bd2[c], pk(-inv[0], -inv[1])));   // dL/dalpha
-    float wv[2];
-    upk(mul2(AL, T2[c]), wv[0], wv[1]);
-    wv[0] = select_f(act[0], wv[0], 0.f);
-    wv[1] = select_f(act[1], wv[1], 0.f);
-    const f2 w = pk(wv[0], wv[1]);
+    const f2 w = mul2(AL, T2[c]);
     Bd2[c] = fma2(cd, w, Bd2[c]);
-    const f2 gd = mul2(pk(select_f(live[0], G[0], 0.f), select_f(live[1], G[1], 0.f)), dal);
-    const f2 dpow = mul2(O2, gd);                       // dL/d(power), natural units
+    f2 dpow;                                            // dL/d(power), natural units
+    if constexpr (kClamp) {
+      // alpha = 0.99 is constant in the splat's parameters
+      dpow = mul2(pk(select_f(raw[0] > kAlphaMax, 0.f, al[0]), select_f(raw[1] > kAlphaMax, 0.f, al[1])),
+                  dal);
+    } else {
+      dpow = mul2(AL, dal);
+    }
     const f2 pdy = mul2(dpow, dy);
-    g4 = fma2(pdy, dy, g4);
-    g5 = add2(g5, gd);
-    g6 = fma2(w, Q0[c], g6);
-    g7 = fma2(w, Q1[c], g7);
-    g8 = fma2(w, Q2[c], g8);
+    pdy_all = c == 0 ? pdy : add2(pdy_all, pdy);
+    w0 = c == 0 ? mul2(w, Q0[c]) : fma2(w, Q0[c], w0);
+    w1 = c == 0 ? mul2(w, Q1[c]) : fma2(w, Q1[c], w1);
+    w2 = c == 0 ? mul2(w, Q2[c]) : fma2(w, Q2[c], w2);
     // the column's sums of dpow and dpow * dy (dx is shared by its rows)
-    float dp[2], pd[2];
-    upk(dpow, dp[0], dp[1]);
-    upk(pdy, pd[0], pd[1]);
-    const float D = dp[0] + dp[1];
-    const float E = fmaf(dp[1], dyv[1], pd[0]);
-    float dx, dxh;
-    upk(dx2, dx, dxh);
-    const float t = dx * D;
-    g[0] += t;
-    g[1] += E;
-    g[2] = fmaf(t, dx, g[2]);
-    g[3] = fmaf(dx, E, g[3]);
+    float x, y;
+    upk(dpow, x, y);
+    D[c] = x + y;
+    upk(pdy, x, y);
+    E[c] = x + y;
+    upk(dx2, dx[c], x);
   }
+  const float t0 = dx[0] * D[0], t1 = dx[1] * D[1];
+  g[0] = t0 + t1;
+  g[1] = E[0] + E[1];
+  g[2] = fmaf(t1, dx[1], t0 * dx[0]);
+  g[3] = fmaf(dx[1], E[1], dx[0] * E[0]);
+  g[5] = D[0] + D[1];
+  float x, y;
+  upk(mul2(pdy_all, dy), x, y);
+  g[4] = x + y;
+  upk(w0, x, y);
+  g[6] = x + y;
+  upk(w1, x, y);
+  g[7] = x + y;
+  upk(w2, x, y);
+  g[8] = x + y;
+}
+
+// Warp sums of the nine values of two splats through shared memory. Each lane
+// stores its nine shares of a splat as one column of nine rows of 32 (pitch
+// 36 words: the stores and the row reads below are both free of bank
+// conflicts). Once two splats are stored, lane l sums half (16 floats, four
+// 128-bit loads, packed adds) of row (l / 2) of the sixteen rows of values
+// 0..7, and 16 lanes per splat share the row of value 8. That is 18 stores, 5
+// loads and about 14 additions and shuffles per two splats, where a butterfly
+// with transposition took 14 shuffles, 14 selects and 14 additions per splat
+// (plus its latency of five dependent shuffles). With the alpha-0 form of
+// bwd_splat the kernel went from 1.793 to 1.689 ms at the surround rig (1.05G
+// evaluated pairs) and from 0.330 to 0.315 ms on one 1080p view; two resident
+// CTAs fewer per SM (72 registers, no spills) took 1.758 and 0.319 ms.
+constexpr int kSumPitch = 36;
+constexpr int kSumSlot = 9 * kSumPitch;           // words per splat
+constexpr int kSumWords = 2 * kSumSlot;           // words per warp
+
+__device__ __forceinline__ void sum_store(float* col, const float (&g)[9]) {
+#pragma unroll
+  for (int v = 0; v < 9; ++v) col[v * kSumPitch] = g[v];
+}
+
+// `half_row` and `ninth` are this lane's read positions (see sum_positions).
+// On return, even lanes hold the total of value (l / 2) % 8 of splat l / 16 in
+// `tot`, and every lane the total of value 8 of splat l / 16 in `tot9`.
+__device__ __forceinline__ void sum_rows(const float* half_row, const float* ninth, float& tot,
+                                         float& tot9) {
+  const float4* h = reinterpret_cast<const float4*>(half_row);
+  const float4 a = h[0], b = h[1], c = h[2], d = h[3];
+  const float2 e = *reinterpret_cast<const float2*>(ninth);
+  const f2 ab = add2(add2(pk(a.x, a.y), pk(a.z, a.w)), add2(pk(b.x, b.y), pk(b.z, b.w)));
+  const f2 cd = add2(add2(pk(c.x, c.y), pk(c.z, c.w)), add2(pk(d.x, d.y), pk(d.z, d.w)));
+  float x, y;
+  upk(add2(ab, cd), x, y);
+  tot = x + y;
+  tot += __shfl_xor_sync(0xffffffffu, tot, 1);
+  tot9 = e.x + e.y;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) tot9 += __shfl_xor_sync(0xffffffffu, tot9, o);
 }
 
 // The reverse walk evaluates a lane's two pixels of a column (rows y and
@@ -825,6 +868,7 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
   __shared__ uint32_t s_id[kBatchBwd];
   __shared__ float s_g[kBatchBwd][9];
   __shared__ float s_sink[kBandThreads];   // target of the lanes with no sum to add
+  __shared__ __align__(16) float s_sum[kBandWarps][kSumWords];
   __shared__ int s_max;
   __shared__ uint32_t s_cstart[kTileClasses + 2];
   __shared__ int s_tile;
@@ -883,6 +927,13 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
     __syncthreads();
     const int n = s_max;
     uint32_t n_eval = 0;   // counting mode: pairs inside their pixel's walk
+    // the lane's column, half row and ninth-row positions of the warp's sums
+    float* sum_col = s_sum[warp] + lane;
+    const float* sum_half = s_sum[warp] + (lane >> 4) * kSumSlot + ((lane >> 1) & 7u) * kSumPitch +
+                            (lane & 1u) * 16u;
+    const float* sum_ninth = s_sum[warp] + (lane >> 4) * kSumSlot + 8 * kSumPitch + (lane & 15u) * 2u;
+    const int sum_value = (lane & 1u) ? 8 : (int)((lane >> 1) & 7u);
+    const bool sum_owner = (lane & 1u) == 0 || (lane & 15u) == 1u;
     // the forward recorded its contributors per band, with the same bands
     const uint32_t* wbits = a.contrib + warp * a.contrib_words;
 
@@ -918,6 +969,8 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
         if (span < 32) todo &= (1u << span) - 1u;
         // as a ballot result the mask is warp-uniform to the compiler as well
         todo = __ballot_sync(0xffffffffu, (todo >> lane) & 1u);
+        int jA = 0;
+        bool second = false;   // the slot of the next splat
         while (todo) {
           const int bit = 31 - __clz(todo);
           todo &= ~(1u << bit);
@@ -925,34 +978,31 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
           const float4 q0 = s_p0[j], q1 = s_p1[j], q2 = s_p2[j], q3 = s_p3[j];
           const float2 qu = s_u[j];
           const int pos = lo + j;
-          float g[4];
-          f2 g4, g5, g6, g7, g8;
+          float g[9];
           // warp-uniform: every lane walks the same splat
           if (q1.z > kAlphaMax)
             bwd_splat<kCount, true>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, last, T2, Bd2, Q0, Q1, Q2,
-                                    n_eval, g, g4, g5, g6, g7, g8);
+                                    n_eval, g);
           else
             bwd_splat<kCount, false>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, last, T2, Bd2, Q0, Q1, Q2,
-                                     n_eval, g, g4, g5, g6, g7, g8);
-          float gs[9] = {g[0], g[1], g[2], g[3], 0.f, 0.f, 0.f, 0.f, 0.f};
-          {
-            float lo4, hi4;
-            upk(g4, lo4, hi4); gs[4] = lo4 + hi4;
-            upk(g5, lo4, hi4); gs[5] = lo4 + hi4;
-            upk(g6, lo4, hi4); gs[6] = lo4 + hi4;
-            upk(g7, lo4, hi4); gs[7] = lo4 + hi4;
-            upk(g8, lo4, hi4); gs[8] = lo4 + hi4;
+                                     n_eval, g);
+          sum_store(sum_col + (second ? kSumSlot : 0), g);
+          if (!second) jA = j;
+          if (second || todo == 0) {
+            __syncwarp();
+            float tot, tot9;
+            sum_rows(sum_half, sum_ninth, tot, tot9);
+            // one shared atomic per warp and two splats: even lanes add value
+            // (l / 2) % 8, lanes 1 and 17 the ninth, the rest (and the second
+            // splat's lanes where there is none) to their own sink word
+            const bool high = lane >= 16u;
+            float* dst = s_g[high ? j : jA] + sum_value;
+            const bool own = sum_owner && (second || !high);
+            dst = own ? dst : &s_sink[threadIdx.x];
+            red_shared(dst, select_f((lane & 1u) == 0, tot, tot9));
+            __syncwarp();   // the rows are rewritten
           }
-          const float tot = warp_sum8_transposed(gs, lane);
-          float g8s = gs[8];
-  #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) g8s += __shfl_xor_sync(0xffffffffu, g8s, o);
-          // one shared atomic per warp: lanes 4m add value m, lane 1 the ninth
-          // sum, the rest add to their own sink word. Predicated atomics compiled
-          // to divergent branches (two per splat).
-          const bool own = (lane & 3u) == 0;
-          float* dst = own ? &s_g[j][lane >> 2] : (lane == 1 ? &s_g[j][8] : &s_sink[threadIdx.x]);
-          red_shared(dst, select_f(own, tot, g8s));
+          second = !second;
         }
       }
       __syncthreads();
@@ -969,7 +1019,7 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
           const float gu = kLn2 * fmaf(2.f * A2, sg[0], B2 * sg[1]);
           const float gv = kLn2 * fmaf(B2, sg[0], 2.f * C2 * sg[1]);
           red_v4(dst, gu, gv, -0.5f * sg[2], -sg[3]);
-          red_v4(dst + 4, -0.5f * sg[4], sg[5], sg[6], sg[7]);
+          red_v4(dst + 4, -0.5f * sg[4], __fdividef(sg[5], s_p1[i].z), sg[6], sg[7]);
           atomicAdd(dst + 8, sg[8]);
         }
       }
