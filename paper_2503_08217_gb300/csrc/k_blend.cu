@@ -40,7 +40,7 @@ namespace {
 #define S3R_BLEND_BWD_BATCH 64    // splats staged per batch (backward)
 #endif
 #ifndef S3R_BLEND_BWD_BLOCKS
-#define S3R_BLEND_BWD_BLOCKS 16   // resident backward blocks per SM (register budget)
+#define S3R_BLEND_BWD_BLOCKS 14   // resident backward blocks per SM (register budget)
 #endif
 
 constexpr int kBatchBwd = S3R_BLEND_BWD_BATCH;
@@ -250,40 +250,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-// Two FP32 values in one 64-bit register for the packed .f32x2 instructions
-// (sm_100 and later): one instruction does the same IEEE operation on both
-// halves, so the pixel pairs of a lane cost half the issue slots of scalar
-// code with bit-identical results.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 pk(float a, float b) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void upk(f2 v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-  f2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
-  f2 d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-  f2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-  f2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
 }
 
 // Shared-memory form of a splat for the blend: the conic is pre-scaled so that
@@ -657,19 +623,17 @@ __device__ __forceinline__ float select_f(bool a, float x, float y) {
   return r;
 }
 
-// The backward's decision for one pixel as one predicate chain: the splat's
-// alpha where the forward blended it (position before the pixel's last
-// contributor, p <= 0, alpha >= 1/255), else 0.
-__device__ __forceinline__ float taken_alpha(float p, float al, int pos, int last) {
-  float r;
+// The backward's decision for one pixel as one predicate chain: G is kept where
+// the forward blended the splat (position before the pixel's last contributor,
+// p <= 0, alpha >= 1/255) and becomes 0 elsewhere.
+__device__ __forceinline__ void keep_taken(float p, float al, float& G, int pos, int last) {
   asm("{\n\t.reg .pred q;\n\t"
       "setp.lt.s32 q, %3, %4;\n\t"
-      "setp.leu.and.f32 q, %1, 0f00000000, q;\n\t"
-      "setp.geu.and.f32 q, %2, %5, q;\n\t"
-      "selp.f32 %0, %2, 0f00000000, q;\n\t}"
-      : "=f"(r)
-      : "f"(p), "f"(al), "r"(pos), "r"(last), "f"(kAlphaMin));
-  return r;
+      "setp.leu.and.f32 q, %2, 0f00000000, q;\n\t"
+      "setp.geu.and.f32 q, %1, %5, q;\n\t"
+      "selp.f32 %0, %0, 0f00000000, q;\n\t}"
+      : "+f"(G)
+      : "f"(al), "f"(p), "r"(pos), "r"(last), "f"(kAlphaMin));
 }
 
 __device__ __forceinline__ void red_shared(float* addr, float v) {
@@ -724,11 +688,12 @@ __device__ __forceinline__ void bwd_init(BwdPixel& q, const BlendArgs& a, const 
 // pixel pairs: updates T and Bd, returns the lane's shares of the nine sums in
 // g. kClamp as for fwd_splat, per splat.
 //
-// A pixel that does not take the splat gets alpha 0: 1 / (1 - 0) is exactly 1,
-// so T, the weight and every sum are left unchanged by the same arithmetic,
-// with one select per pixel. Without the cap, alpha = o G, so G dL/dalpha (the
-// opacity's term) is (alpha dL/dalpha) / o and the sum of the power's adjoint
-// serves both; the division is made once per splat at the flush.
+// A pixel that does not take the splat gets G = 0, hence alpha 0: 1 / (1 - 0) is
+// exactly 1, so T, the weight and every sum are left unchanged by the same
+// arithmetic, with one select per pixel. A thin splat's moments cancel in the
+// chain to its covariance, which magnifies their last bits by the splat's
+// aspect ratio, so the sums' order of additions is kept fixed (here and in
+// sum_rows).
 template <bool kCount, bool kClamp>
 __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, const float4 q2,
                                           const float4 q3, const float2 qu, const f2 FY,
@@ -743,23 +708,32 @@ __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, cons
   const f2 dy = sub2(V2, FY);
   const f2 bdy = mul2(B2, dy);
   const f2 cdy = mul2(mul2(C2c, dy), dy);
-  f2 pdy_all, w0, w1, w2;
-  float D[2], E[2], dx[2];
+  f2 gdy, gop, w0, w1, w2;
+  float D[2], E[2], dx[2], dyv[2], x, y;
+  upk(dy, dyv[0], dyv[1]);
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const f2 dx2 = sub2(U2, FX[c]);
     const f2 pw = fma2(dx2, fma2(A2, dx2, bdy), cdy);
-    float p[2], raw[2], al[2], inv[2];
+    float p[2], G[2], raw[2], inv[2];
     upk(pw, p[0], p[1]);
-    upk(mul2(O2, pk(ex2_approx(p[0]), ex2_approx(p[1]))), raw[0], raw[1]);
+    G[0] = ex2_approx(p[0]);
+    G[1] = ex2_approx(p[1]);
+    upk(mul2(O2, pk(G[0], G[1])), raw[0], raw[1]);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int k = c * kRows + r;
-      al[r] = kClamp ? fminf(kAlphaMax, raw[r]) : raw[r];
       if constexpr (kCount) n_eval += pos < last[k] ? 1u : 0u;
-      al[r] = taken_alpha(p[r], al[r], pos, last[k]);
+      keep_taken(p[r], kClamp ? fminf(kAlphaMax, raw[r]) : raw[r], G[r], pos, last[k]);
     }
-    const f2 AL = pk(al[0], al[1]);
+    f2 AL = mul2(O2, pk(G[0], G[1]));
+    if constexpr (kClamp) {
+      // alpha = 0.99 is constant in the splat's parameters
+      upk(AL, x, y);
+      AL = pk(fminf(kAlphaMax, x), fminf(kAlphaMax, y));
+      G[0] = select_f(x > kAlphaMax, 0.f, G[0]);
+      G[1] = select_f(y > kAlphaMax, 0.f, G[1]);
+    }
     upk(sub2(ONE, AL), inv[0], inv[1]);
     inv[0] = rcp_approx(inv[0]);
     inv[1] = rcp_approx(inv[1]);
@@ -769,25 +743,20 @@ __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, cons
     const f2 dal = fma2(T2[c], cd, mul2(Bd2[c], pk(-inv[0], -inv[1])));   // dL/dalpha
     const f2 w = mul2(AL, T2[c]);
     Bd2[c] = fma2(cd, w, Bd2[c]);
-    f2 dpow;                                            // dL/d(power), natural units
-    if constexpr (kClamp) {
-      // alpha = 0.99 is constant in the splat's parameters
-      dpow = mul2(pk(select_f(raw[0] > kAlphaMax, 0.f, al[0]), select_f(raw[1] > kAlphaMax, 0.f, al[1])),
-                  dal);
-    } else {
-      dpow = mul2(AL, dal);
-    }
+    const f2 gd = mul2(pk(G[0], G[1]), dal);
+    const f2 dpow = mul2(O2, gd);                       // dL/d(power), natural units
     const f2 pdy = mul2(dpow, dy);
-    pdy_all = c == 0 ? pdy : add2(pdy_all, pdy);
+    gdy = c == 0 ? mul2(pdy, dy) : fma2(pdy, dy, gdy);
+    gop = c == 0 ? gd : add2(gop, gd);
     w0 = c == 0 ? mul2(w, Q0[c]) : fma2(w, Q0[c], w0);
     w1 = c == 0 ? mul2(w, Q1[c]) : fma2(w, Q1[c], w1);
     w2 = c == 0 ? mul2(w, Q2[c]) : fma2(w, Q2[c], w2);
     // the column's sums of dpow and dpow * dy (dx is shared by its rows)
-    float x, y;
-    upk(dpow, x, y);
-    D[c] = x + y;
+    float dp0, dp1;
+    upk(dpow, dp0, dp1);
     upk(pdy, x, y);
-    E[c] = x + y;
+    D[c] = dp0 + dp1;
+    E[c] = fmaf(dp1, dyv[1], x);
     upk(dx2, dx[c], x);
   }
   const float t0 = dx[0] * D[0], t1 = dx[1] * D[1];
@@ -795,10 +764,10 @@ __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, cons
   g[1] = E[0] + E[1];
   g[2] = fmaf(t1, dx[1], t0 * dx[0]);
   g[3] = fmaf(dx[1], E[1], dx[0] * E[0]);
-  g[5] = D[0] + D[1];
-  float x, y;
-  upk(mul2(pdy_all, dy), x, y);
+  upk(gdy, x, y);
   g[4] = x + y;
+  upk(gop, x, y);
+  g[5] = x + y;
   upk(w0, x, y);
   g[6] = x + y;
   upk(w1, x, y);
@@ -812,13 +781,17 @@ __device__ __forceinline__ void bwd_splat(const float4 q0, const float4 q1, cons
 // 36 words: the stores and the row reads below are both free of bank
 // conflicts). Once two splats are stored, lane l sums half (16 floats, four
 // 128-bit loads, packed adds) of row (l / 2) of the sixteen rows of values
-// 0..7, and 16 lanes per splat share the row of value 8. That is 18 stores, 5
+// 0..7, and 16 lanes per splat share the row of value 8. That is 18 stores, 6
 // loads and about 14 additions and shuffles per two splats, where a butterfly
 // with transposition took 14 shuffles, 14 selects and 14 additions per splat
-// (plus its latency of five dependent shuffles). With the alpha-0 form of
-// bwd_splat the kernel went from 1.793 to 1.689 ms at the surround rig (1.05G
-// evaluated pairs) and from 0.330 to 0.315 ms on one 1080p view; two resident
-// CTAs fewer per SM (72 registers, no spills) took 1.758 and 0.319 ms.
+// (plus its latency of five dependent shuffles). The columns stand in the order
+// (even lanes, odd lanes), so that the halves' sums pair lanes 16, 8, 4, 2
+// and 1 apart, in that order, as the butterfly does: the totals have its bits.
+// At 14 CTAs per SM (72 registers) one 1080p view's backward went from 0.330 to
+// 0.321 ms and a 1001 x 563 view's from 0.083 to 0.081 ms; the surround rig
+// (1.05G evaluated pairs) stayed at 1.79 ms, where a packed FMA costs the
+// issue slots of two scalar ones and the shuffles had hidden behind them. 16
+// CTAs (64 registers) took 0.332 and 1.785 ms, 12 (80) 0.328 and 1.850 ms.
 constexpr int kSumPitch = 36;
 constexpr int kSumSlot = 9 * kSumPitch;           // words per splat
 constexpr int kSumWords = 2 * kSumSlot;           // words per warp
@@ -828,21 +801,20 @@ __device__ __forceinline__ void sum_store(float* col, const float (&g)[9]) {
   for (int v = 0; v < 9; ++v) col[v * kSumPitch] = g[v];
 }
 
-// `half_row` and `ninth` are this lane's read positions (see sum_positions).
-// On return, even lanes hold the total of value (l / 2) % 8 of splat l / 16 in
-// `tot`, and every lane the total of value 8 of splat l / 16 in `tot9`.
+// `half_row` and `ninth` are this lane's read positions. On return, even lanes
+// hold the total of value (l / 2) % 8 of splat l / 16 in `tot`, and every lane
+// the total of value 8 of splat l / 16 in `tot9`.
 __device__ __forceinline__ void sum_rows(const float* half_row, const float* ninth, float& tot,
                                          float& tot9) {
   const float4* h = reinterpret_cast<const float4*>(half_row);
   const float4 a = h[0], b = h[1], c = h[2], d = h[3];
-  const float2 e = *reinterpret_cast<const float2*>(ninth);
-  const f2 ab = add2(add2(pk(a.x, a.y), pk(a.z, a.w)), add2(pk(b.x, b.y), pk(b.z, b.w)));
-  const f2 cd = add2(add2(pk(c.x, c.y), pk(c.z, c.w)), add2(pk(d.x, d.y), pk(d.z, d.w)));
+  const f2 lo = add2(add2(pk(a.x, a.y), pk(c.x, c.y)), add2(pk(b.x, b.y), pk(d.x, d.y)));
+  const f2 hi = add2(add2(pk(a.z, a.w), pk(c.z, c.w)), add2(pk(b.z, b.w), pk(d.z, d.w)));
   float x, y;
-  upk(add2(ab, cd), x, y);
+  upk(add2(lo, hi), x, y);
   tot = x + y;
   tot += __shfl_xor_sync(0xffffffffu, tot, 1);
-  tot9 = e.x + e.y;
+  tot9 = ninth[0] + ninth[8];
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) tot9 += __shfl_xor_sync(0xffffffffu, tot9, o);
 }
@@ -928,10 +900,11 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
     const int n = s_max;
     uint32_t n_eval = 0;   // counting mode: pairs inside their pixel's walk
     // the lane's column, half row and ninth-row positions of the warp's sums
-    float* sum_col = s_sum[warp] + lane;
+    float* sum_col = s_sum[warp] + (lane & 1u) * 16u + (lane >> 1);
     const float* sum_half = s_sum[warp] + (lane >> 4) * kSumSlot + ((lane >> 1) & 7u) * kSumPitch +
                             (lane & 1u) * 16u;
-    const float* sum_ninth = s_sum[warp] + (lane >> 4) * kSumSlot + 8 * kSumPitch + (lane & 15u) * 2u;
+    const float* sum_ninth = s_sum[warp] + (lane >> 4) * kSumSlot + 8 * kSumPitch + (lane & 1u) * 16u +
+                             ((lane & 15u) >> 1);
     const int sum_value = (lane & 1u) ? 8 : (int)((lane >> 1) & 7u);
     const bool sum_owner = (lane & 1u) == 0 || (lane & 15u) == 1u;
     // the forward recorded its contributors per band, with the same bands
@@ -1019,7 +992,7 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
           const float gu = kLn2 * fmaf(2.f * A2, sg[0], B2 * sg[1]);
           const float gv = kLn2 * fmaf(B2, sg[0], 2.f * C2 * sg[1]);
           red_v4(dst, gu, gv, -0.5f * sg[2], -sg[3]);
-          red_v4(dst + 4, -0.5f * sg[4], __fdividef(sg[5], s_p1[i].z), sg[6], sg[7]);
+          red_v4(dst + 4, -0.5f * sg[4], sg[5], sg[6], sg[7]);
           atomicAdd(dst + 8, sg[8]);
         }
       }
@@ -1096,7 +1069,7 @@ cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cu
     // pairs walked and evaluated (two adjacent 64-bit counters)
     if ((e = cudaMemsetAsync(a.pairs, 0, 2 * sizeof(unsigned long long), st)) != cudaSuccess) return e;
   }
-  // the contributor bits were cleared by the sort's tile ranges
+  // the contributor bits were cleared by the sort's pair expansion
   static thread_local int per_sm[2] = {0, 0};
   KernelTimer timer(ws, kKBlendFwd, st);
   if (ws->counting) {
