@@ -7,14 +7,28 @@
 // a unit quaternion with the translation z[0:3] (the instance pose of
 // Sec. 3.3, local -> world).
 //
-// One warp per instance, all instances in parallel; the time steps of an
-// instance are sequential. Lane l holds hidden units l and l + 32. The
-// weights sit in shared memory in the layouts the lanes read without bank
-// conflicts (W1 and W2 transposed for the forward, W2 also row-major for the
-// backward's W2^T product). The backward walks an instance's steps in
-// reverse from the stored states, recomputes each step's four stages and
-// accumulates the parameter adjoints in per-warp copies in shared memory,
-// summed over the CTA's warps and added to the caller's buffer at the end.
+// An instance's time steps are a chain of dependent evaluations of f, so the
+// kernels are bound by the latency of one evaluation, not by throughput. One
+// evaluation is spread over a group of two warps, thread u owning hidden unit
+// u with its rows of the weights in registers; the 64-wide hidden vectors are
+// exchanged through shared memory (one store, one 64-thread barrier, sixteen
+// broadcast 128-bit loads) and the dot products are packed f32x2 FMAs in four
+// chains. The six outputs are taken by four lanes each and broadcast with
+// shuffles. With one warp per instance, two units per lane and the weights read
+// from shared memory, an evaluation took about 2,200 cycles.
+//
+// The backward walks an instance's steps in reverse from the stored states. Its
+// chain is only the adjoint: recomputing a step's four stages does not depend on
+// it, nor do the parameter sums feed it. So a CTA (one instance) runs four
+// groups side by side, two steps per tick: two groups recompute the stages of
+// the tick's two steps, a third walks the adjoint through the two steps
+// recomputed one tick earlier, a fourth adds the parameter adjoints of the two
+// steps walked before those, its rows of the sums in registers. They meet at
+// one CTA barrier per tick and pass the activations through a ring of three
+// ticks in shared memory.
+//
+// At 120 instances, 400 times, 2 substeps and embedding width 8 the forward and
+// the backward together went from 15.1 to 2.27 ms.
 #include "s3r_internal.cuh"
 
 namespace s3r {
@@ -22,8 +36,8 @@ namespace {
 
 constexpr int kH = S3R_ODE_HIDDEN;     // hidden width
 constexpr int kMaxD = S3R_ODE_MAX_EMBED;
-constexpr int kOdeWarps = 4;           // instances per CTA
-static_assert(kH == 64, "lanes hold hidden units l and l + 32");
+constexpr int kGroup = kH;             // threads of a group: one per hidden unit
+static_assert(kGroup == 64, "a group is two warps");
 
 struct OdeLayout {
   int D, I;
@@ -43,87 +57,95 @@ __host__ __device__ inline OdeLayout ode_layout(int D) {
   return L;
 }
 
-// Shared weights: W1t [I][H] (W1t[i][u] = W1[u][i]), b1 [H], W2t [H][H]
-// (W2t[j][u] = W2[u][j]), W2 [H][H], b2 [H], W3 [6][H], b3 [6].
-struct SW {
-  float* W1t;
-  float* b1;
-  float* W2t;
-  float* W2;
-  float* b2;
-  float* W3;
-  float* b3;
-};
-__host__ __device__ inline int sw_floats(int I) { return I * kH + kH + 2 * kH * kH + kH + 6 * kH + 6; }
-
-__device__ SW load_weights(const float* __restrict__ p, const OdeLayout& L, float* smem) {
-  SW w;
-  w.W1t = smem;
-  w.b1 = w.W1t + L.I * kH;
-  w.W2t = w.b1 + kH;
-  w.W2 = w.W2t + kH * kH;
-  w.b2 = w.W2 + kH * kH;
-  w.W3 = w.b2 + kH;
-  w.b3 = w.W3 + 6 * kH;
-  for (int e = threadIdx.x; e < kH * L.I; e += blockDim.x) {
-    const int u = e / L.I, i = e - u * L.I;
-    w.W1t[i * kH + u] = p[L.oW1 + e];
-  }
-  for (int e = threadIdx.x; e < kH * kH; e += blockDim.x) {
-    const int u = e / kH, j = e - u * kH;
-    const float v = p[L.oW2 + e];
-    w.W2t[j * kH + u] = v;
-    w.W2[e] = v;
-  }
-  for (int e = threadIdx.x; e < kH; e += blockDim.x) {
-    w.b1[e] = p[L.ob1 + e];
-    w.b2[e] = p[L.ob2 + e];
-  }
-  for (int e = threadIdx.x; e < 6 * kH; e += blockDim.x) w.W3[e] = p[L.oW3 + e];
-  for (int e = threadIdx.x; e < 6; e += blockDim.x) w.b3[e] = p[L.ob3 + e];
-  return w;
+// Barrier of one group (two warps); ids 1..4, 0 is the CTA's.
+__device__ __forceinline__ void group_sync(int id) {
+  asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
 }
 
-__device__ __forceinline__ float warp_sum(float v) {
+// Sum over the 64 entries of `v` (shared memory, 16-byte aligned) of v[m] w[m],
+// w as consecutive pairs in registers.
+__device__ __forceinline__ float dot64(const float* v, const f2 (&w)[kH / 2]) {
+  const float4* v4 = reinterpret_cast<const float4*>(v);
+  f2 acc[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// f(z, t, c) (Eq. 3) for the warp's instance: `out` (6, the same in every
-// lane) and the lane's hidden activations h1[2], h2[2] (units l, l + 32).
-__device__ __forceinline__ void eval_f(const SW& w, int I, const float (&z)[6], float t,
-                                       const float* c, int D, uint32_t lane, float (&out)[6],
-                                       float (&h1)[2], float (&h2)[2]) {
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int u = (int)lane + 32 * q;
-    float a = w.b1[u];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) a = fmaf(w.W1t[i * kH + u], z[i], a);
-    a = fmaf(w.W1t[6 * kH + u], t, a);
-    for (int d = 0; d < D; ++d) a = fmaf(w.W1t[(7 + d) * kH + u], c[d], a);
-    h1[q] = tanhf(a);
-  }
-  // four partial sums per output (inputs j = 4 i + p), so that the chain of
-  // dependent FMAs is 16 long instead of 64: the products are latency-bound
-  // (one warp per instance walks its steps in sequence)
-  float a0[4] = {w.b2[lane], 0.f, 0.f, 0.f}, a1[4] = {w.b2[lane + 32], 0.f, 0.f, 0.f};
-#pragma unroll 4
   for (int i = 0; i < kH / 4; ++i) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int j = 4 * i + q;
-      const float hj = __shfl_sync(0xffffffffu, h1[j >> 5], j & 31);
-      a0[q] = fmaf(w.W2t[j * kH + lane], hj, a0[q]);
-      a1[q] = fmaf(w.W2t[j * kH + lane + 32], hj, a1[q]);
-    }
+    const float4 x = v4[i];
+    const int q = 2 * (i & 1);
+    const f2 lo = pk(x.x, x.y), hi = pk(x.z, x.w);
+    acc[q] = i < 2 ? mul2(lo, w[2 * i]) : fma2(lo, w[2 * i], acc[q]);
+    acc[q + 1] = i < 2 ? mul2(hi, w[2 * i + 1]) : fma2(hi, w[2 * i + 1], acc[q + 1]);
   }
-  h2[0] = tanhf((a0[0] + a0[1]) + (a0[2] + a0[3]));
-  h2[1] = tanhf((a1[0] + a1[1]) + (a1[2] + a1[3]));
+  float a, b;
+  upk(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), a, b);
+  return a + b;
+}
+
+// Six 64-term sums at once: lane 4 o + q (o < 6) takes the 16 terms of output o
+// in the float4s q, q + 4, q + 8, q + 12 of v; two shuffles add the quarters and
+// six broadcast the outputs to every lane. `first` is added to output o.
+__device__ __forceinline__ void six_sums(const float* v, const f2 (&w)[8], float first, uint32_t lane,
+                                         float (&out)[6]) {
+  const float4* v4 = reinterpret_cast<const float4*>(v) + (lane & 3u);
+  f2 acc[2];
 #pragma unroll
-  for (int o = 0; o < 6; ++o)
-    out[o] = w.b3[o] + warp_sum(fmaf(w.W3[o * kH + lane], h2[0], w.W3[o * kH + lane + 32] * h2[1]));
+  for (int i = 0; i < 4; ++i) {
+    const float4 x = v4[4 * i];
+    acc[0] = i == 0 ? mul2(pk(x.x, x.y), w[0]) : fma2(pk(x.x, x.y), w[2 * i], acc[0]);
+    acc[1] = i == 0 ? mul2(pk(x.z, x.w), w[1]) : fma2(pk(x.z, x.w), w[2 * i + 1], acc[1]);
+  }
+  float a, b;
+  upk(add2(acc[0], acc[1]), a, b);
+  a += b;
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  a += first;
+#pragma unroll
+  for (int o = 0; o < 6; ++o) out[o] = __shfl_sync(0xffffffffu, a, 4 * o);
+}
+
+// Weights of one evaluation of f that thread u of a group keeps in registers.
+struct EvalWeights {
+  f2 w2[kH / 2];        // row u of W2
+  f2 w3[8];             // its lane's quarter of row lane / 4 of W3 (see six_sums)
+  float w1[6], wt;      // row u of W1: z and t
+  float base;           // b1[u] + W1[u, 7:] c
+  float b2, b3;
+};
+__device__ __forceinline__ void load_eval_weights(EvalWeights& e, const float* __restrict__ p,
+                                                  const OdeLayout& L, const float* c, int u) {
+  const uint32_t lane = (uint32_t)u & 31u;
+  const float* W1 = p + L.oW1 + (int64_t)u * L.I;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) e.w1[i] = W1[i];
+  e.wt = W1[6];
+  e.base = p[L.ob1 + u];
+  for (int d = 0; d < L.D; ++d) e.base = fmaf(W1[7 + d], c[d], e.base);
+  const float* W2 = p + L.oW2 + (int64_t)u * kH;
+#pragma unroll
+  for (int m = 0; m < kH / 2; ++m) e.w2[m] = pk(W2[2 * m], W2[2 * m + 1]);
+  e.b2 = p[L.ob2 + u];
+  const int o = (int)(lane >> 2);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int m = 4 * ((int)(lane & 3u) + 4 * (i >> 1)) + 2 * (i & 1);
+    e.w3[i] = o < 6 ? pk(p[L.oW3 + o * kH + m], p[L.oW3 + o * kH + m + 1]) : pk(0.f, 0.f);
+  }
+  e.b3 = o < 6 ? p[L.ob3 + o] : 0.f;
+}
+
+// f(z, t, c) (Eq. 3) by one group: `out` in every thread; the hidden activations
+// go to h1 and h2 (64 floats of shared memory each). h1 may be rewritten by the
+// next evaluation and h2 after the next evaluation's first barrier, which is
+// where this function writes them, so evaluations follow each other freely.
+__device__ __forceinline__ void eval_f(const EvalWeights& e, const float (&z)[6], float t, int u,
+                                       int bar, float* h1, float* h2, float (&out)[6]) {
+  const float a = fmaf(e.w1[2], z[2], fmaf(e.w1[1], z[1], fmaf(e.w1[0], z[0], fmaf(e.wt, t, e.base))));
+  const float b = fmaf(e.w1[5], z[5], fmaf(e.w1[4], z[4], e.w1[3] * z[3]));
+  h1[u] = tanhf(a + b);
+  group_sync(bar);
+  h2[u] = tanhf(dot64(h1, e.w2) + e.b2);
+  group_sync(bar);
+  six_sums(h2, e.w3, e.b3, (uint32_t)u & 31u, out);
 }
 
 // exp(r) as a unit quaternion (w, x, y, z); a series below |r| = 1e-4.
@@ -164,24 +186,6 @@ __device__ __forceinline__ void quat_from_rotvec_vjp(const float r[3], float4 g,
     out[i] = -0.5f * s * r[i] * g.x + s * gv[i] + r[i] * (ds / th) * dot;
 }
 
-__device__ __forceinline__ void store6(float* dst, const float (&v)[6], uint32_t lane) {
-  float x = v[0];
-#pragma unroll
-  for (int i = 1; i < 6; ++i) x = (int)lane == i ? v[i] : x;
-  if (lane < 6) dst[lane] = x;
-}
-
-__device__ __forceinline__ void write_pose(const float (&z)[6], float* quat, float* trans,
-                                           uint32_t lane) {
-  if (lane == 0) {
-    const float4 q = quat_from_rotvec(z[3], z[4], z[5]);
-    *reinterpret_cast<float4*>(quat) = q;
-    trans[0] = z[0];
-    trans[1] = z[1];
-    trans[2] = z[2];
-  }
-}
-
 struct OdeArgs {
   const float* params;
   const float* embed;
@@ -198,252 +202,285 @@ struct OdeArgs {
   float* g_z0;
 };
 
-__global__ void __launch_bounds__(32 * kOdeWarps) k_ode_fwd(OdeArgs a) {
-  extern __shared__ __align__(16) float smem[];
+// One group per instance. The poses come from the stored states once the chain
+// is done, all output times in parallel, so that no sine or cosine sits in it.
+__global__ void __launch_bounds__(kGroup) k_ode_fwd(OdeArgs a) {
+  __shared__ __align__(16) float s_h1[kH], s_h2[kH];
   const OdeLayout L = ode_layout(a.D);
-  const SW w = load_weights(a.params, L, smem);
-  __syncthreads();
-  const uint32_t lane = threadIdx.x & 31u;
-  const int k = blockIdx.x * kOdeWarps + (int)(threadIdx.x >> 5);
-  if (k >= a.n_inst) return;
-  float c[kMaxD];
-  for (int d = 0; d < a.D; ++d) c[d] = a.embed[(size_t)k * a.D + d];
+  const int u = threadIdx.x, k = blockIdx.x, K = a.n_inst;
+  EvalWeights w;
+  load_eval_weights(w, a.params, L, a.embed + (size_t)k * a.D, u);
   float z[6];
 #pragma unroll
   for (int i = 0; i < 6; ++i) z[i] = a.z0[6 * (size_t)k + i];
-  const int K = a.n_inst;
-  store6(a.states + 6 * (size_t)k, z, lane);
-  write_pose(z, a.quat + 4 * (size_t)k, a.trans + 3 * (size_t)k, lane);
-  int step = 0;
+  if (u < 6) a.states[6 * (size_t)k + u] = a.z0[6 * (size_t)k + u];
+  float* dst = a.states + 6 * ((size_t)K + k);
+  float t0 = a.times[0];
   for (int j = 0; j + 1 < a.n_times; ++j) {
-    const float t0 = a.times[j];
-    const float h = (a.times[j + 1] - t0) / (float)a.substeps;
+    const float t1 = a.times[j + 1];
+    const float h = (t1 - t0) / (float)a.substeps;
     for (int s = 0; s < a.substeps; ++s) {
       const float t = t0 + (float)s * h;
-      float k1[6], k2[6], k3[6], k4[6], u[6], h1[2], h2[2];
-      eval_f(w, L.I, z, t, c, a.D, lane, k1, h1, h2);
+      float k1[6], k2[6], k3[6], k4[6], v[6];
+      eval_f(w, z, t, u, 1, s_h1, s_h2, k1);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) u[i] = fmaf(0.5f * h, k1[i], z[i]);
-      eval_f(w, L.I, u, t + 0.5f * h, c, a.D, lane, k2, h1, h2);
+      for (int i = 0; i < 6; ++i) v[i] = fmaf(0.5f * h, k1[i], z[i]);
+      eval_f(w, v, t + 0.5f * h, u, 1, s_h1, s_h2, k2);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) u[i] = fmaf(0.5f * h, k2[i], z[i]);
-      eval_f(w, L.I, u, t + 0.5f * h, c, a.D, lane, k3, h1, h2);
+      for (int i = 0; i < 6; ++i) v[i] = fmaf(0.5f * h, k2[i], z[i]);
+      eval_f(w, v, t + 0.5f * h, u, 1, s_h1, s_h2, k3);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) u[i] = fmaf(h, k3[i], z[i]);
-      eval_f(w, L.I, u, t + h, c, a.D, lane, k4, h1, h2);
+      for (int i = 0; i < 6; ++i) v[i] = fmaf(h, k3[i], z[i]);
+      eval_f(w, v, t + h, u, 1, s_h1, s_h2, k4);
+      float mine = 0.f;
 #pragma unroll
-      for (int i = 0; i < 6; ++i)
+      for (int i = 0; i < 6; ++i) {
         z[i] = fmaf(h * (1.f / 6.f), k1[i] + 2.f * k2[i] + 2.f * k3[i] + k4[i], z[i]);
-      ++step;
-      store6(a.states + 6 * ((size_t)step * K + k), z, lane);
+        mine = u == i ? z[i] : mine;
+      }
+      if (u < 6) dst[u] = mine;
+      dst += 6 * (size_t)K;
     }
-    write_pose(z, a.quat + 4 * ((size_t)(j + 1) * K + k), a.trans + 3 * ((size_t)(j + 1) * K + k),
-               lane);
+    t0 = t1;
+  }
+  __syncthreads();   // the states of this instance are written
+  for (int j = u; j < a.n_times; j += kGroup) {
+    const float* zs = a.states + 6 * ((size_t)j * a.substeps * K + k);
+    const size_t row = (size_t)j * K + k;
+    *reinterpret_cast<float4*>(a.quat + 4 * row) = quat_from_rotvec(zs[3], zs[4], zs[5]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) a.trans[3 * row + i] = zs[i];
   }
 }
 
-// Per-warp adjoint accumulators in shared memory: dW1t [I][H], db1 [H],
-// dW2t [H][H] (dW2t[j][u] = dW2[u][j]), db2 [H], dW3 [6][H], db3 [6].
-__host__ __device__ inline int acc_floats(int I) { return I * kH + kH + kH * kH + kH + 6 * kH + 6; }
-struct Acc {
-  float* W1t;
-  float* b1;
-  float* W2t;
-  float* b2;
-  float* W3;
-  float* b3;
+// What the backward's groups hand to each other for one step: the stages'
+// inputs, activations and times, the adjoints of their outputs and hidden
+// units, and the pose adjoint that enters at the step's end.
+struct __align__(16) StepSlot {
+  float h1[4][kH], h2[4][kH], p1[4][kH], p2[4][kH];
+  float x[4][8];     // z at the stage, then t
+  float yb[4][8];    // adjoint of the stage's output
+  float inj[8];
+  float h;
 };
-__device__ __forceinline__ Acc acc_at(float* base, int I) {
-  Acc g;
-  g.W1t = base;
-  g.b1 = g.W1t + I * kH;
-  g.W2t = g.b1 + kH;
-  g.b2 = g.W2t + kH * kH;
-  g.W3 = g.b2 + kH;
-  g.b3 = g.W3 + 6 * kH;
-  return g;
+static_assert(sizeof(StepSlot) % 16 == 0, "the slots' vectors are read as float4");
+constexpr int kRing = 3, kTickSteps = 2;
+constexpr int kBwdThreads = 4 * kGroup;
+
+// The pose adjoints of state index i (an output time iff i is a multiple of the
+// substeps), for the state's six components.
+__device__ __forceinline__ void pose_adjoint(const OdeArgs& a, int i, int k, float (&g)[6]) {
+#pragma unroll
+  for (int q = 0; q < 6; ++q) g[q] = 0.f;
+  if (i % a.substeps != 0) return;
+  const size_t row = (size_t)(i / a.substeps) * a.n_inst + k;
+  const float* zs = a.states + 6 * ((size_t)i * a.n_inst + k);
+  const float r[3] = {zs[3], zs[4], zs[5]};
+  float gr[3];
+  quat_from_rotvec_vjp(r, *reinterpret_cast<const float4*>(a.g_quat + 4 * row), gr);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    g[q] = a.g_trans[3 * row + q];
+    g[3 + q] = gr[q];
+  }
 }
 
-// VJP of f at one stage: adds the parameter adjoints to the warp's
-// accumulators and returns the adjoints of z (6) and c (D), uniform in lanes.
-__device__ __forceinline__ void vjp_f(const SW& w, const Acc& g, int I, const float (&x6)[6], float t,
-                                      const float* c, int D, const float (&h1)[2],
-                                      const float (&h2)[2], const float (&yb)[6], uint32_t lane,
-                                      float (&zb)[6], float* cb) {
-  // layer 3: dW3 += yb h2^T, db3 += yb, hb2 = W3^T yb
-  float hb2[2] = {0.f, 0.f};
+// Recomputes the stages of step i (from state i - 1 to state i) into its slot.
+__device__ __forceinline__ void recompute_step(const OdeArgs& a, const EvalWeights& w, int i, int k,
+                                               int u, int bar, StepSlot& s) {
+  const int jj = (i - 1) / a.substeps, sub = (i - 1) - jj * a.substeps;
+  const float* zs = a.states + 6 * ((size_t)(i - 1) * a.n_inst + k);
+  float z[6], v[6], kk[6];
 #pragma unroll
-  for (int o = 0; o < 6; ++o) {
-    g.W3[o * kH + lane] += yb[o] * h2[0];
-    g.W3[o * kH + lane + 32] += yb[o] * h2[1];
-    hb2[0] = fmaf(w.W3[o * kH + lane], yb[o], hb2[0]);
-    hb2[1] = fmaf(w.W3[o * kH + lane + 32], yb[o], hb2[1]);
+  for (int q = 0; q < 6; ++q) z[q] = zs[q];
+  const float t0 = a.times[jj];
+  const float h = (a.times[jj + 1] - t0) / (float)a.substeps;
+  const float t = t0 + (float)sub * h;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) v[q] = z[q];
+#pragma unroll
+  for (int st = 0; st < 4; ++st) {
+    const float ts = st == 0 ? t : (st == 3 ? t + h : t + 0.5f * h);
+    if (u < 8) {
+      float mine = ts;
+#pragma unroll
+      for (int q = 0; q < 6; ++q) mine = u == q ? v[q] : mine;
+      s.x[st][u] = mine;
+    }
+    eval_f(w, v, ts, u, bar, s.h1[st], s.h2[st], kk);
+    const float step = st == 2 ? h : 0.5f * h;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v[q] = fmaf(step, kk[q], z[q]);
   }
-  if (lane == 0)
+  if (u == 0) {
+    float g[6];
+    pose_adjoint(a, i, k, g);
 #pragma unroll
-    for (int o = 0; o < 6; ++o) g.b3[o] += yb[o];
-  const float p2[2] = {hb2[0] * (1.f - h2[0] * h2[0]), hb2[1] * (1.f - h2[1] * h2[1])};
-  g.b2[lane] += p2[0];
-  g.b2[lane + 32] += p2[1];
-  // dW2[u][j] += p2[u] h1[j] (lane owns rows u = l, l + 32); hb1[j] = sum_u W2[u][j] p2[u]
-  // (lane owns columns j = l, l + 32)
-  // (four partial sums per column, as in eval_f, to shorten the FMA chain)
-  float hb1a[4] = {0.f, 0.f, 0.f, 0.f}, hb1b[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-  for (int i = 0; i < kH / 4; ++i) {
+    for (int q = 0; q < 6; ++q) s.inj[q] = g[q];
+    s.h = h;
+  }
+}
+
+// Walks the adjoint `ab` of state i back through step i: per stage the reverse
+// of f, hidden layer by hidden layer, with the same exchanges as eval_f.
+struct AdjointWeights {
+  f2 w2[kH / 2];      // column u of W2
+  f2 w1[8];           // its lane's quarter of column lane / 4 of W1 (see six_sums)
+  float w3[6];        // column u of W3
+};
+__device__ __forceinline__ void walk_step(const AdjointWeights& w, int u, int bar, StepSlot& s,
+                                          float (&ab)[6]) {
+  const uint32_t lane = (uint32_t)u & 31u;
+  const float h = s.h;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int m = 4 * i + q;
-      const float h1m = __shfl_sync(0xffffffffu, h1[m >> 5], m & 31);
-      const float p2m = __shfl_sync(0xffffffffu, p2[m >> 5], m & 31);
-      g.W2t[m * kH + lane] += p2[0] * h1m;
-      g.W2t[m * kH + lane + 32] += p2[1] * h1m;
-      hb1a[q] = fmaf(w.W2[m * kH + lane], p2m, hb1a[q]);
-      hb1b[q] = fmaf(w.W2[m * kH + lane + 32], p2m, hb1b[q]);
+  for (int q = 0; q < 6; ++q) ab[q] += s.inj[q];
+  // z' = z + h/6 (k1 + 2 k2 + 2 k3 + k4), stages in reverse
+  float zb[6], kb[6], xb[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    zb[q] = ab[q];
+    kb[q] = h * (1.f / 6.f) * ab[q];
+  }
+#pragma unroll
+  for (int st = 3; st >= 0; --st) {
+    const float h1 = s.h1[st][u], h2 = s.h2[st][u];
+    const float ga = fmaf(w.w3[2], kb[2], fmaf(w.w3[1], kb[1], w.w3[0] * kb[0]));
+    const float gb = fmaf(w.w3[5], kb[5], fmaf(w.w3[4], kb[4], w.w3[3] * kb[3]));
+    s.p2[st][u] = (ga + gb) * (1.f - h2 * h2);
+    if (u < 6) {
+      float mine = 0.f;
+#pragma unroll
+      for (int q = 0; q < 6; ++q) mine = u == q ? kb[q] : mine;
+      s.yb[st][u] = mine;
+    }
+    group_sync(bar);
+    s.p1[st][u] = dot64(s.p2[st], w.w2) * (1.f - h1 * h1);
+    group_sync(bar);
+    six_sums(s.p1[st], w.w1, 0.f, lane, xb);
+    // the next stage's output adjoint: k_st fed the following stage with the
+    // factor `step` and the step's sum with `share`
+    const float step = st == 3 ? h : 0.5f * h;
+    const float share = st == 1 ? h * (1.f / 6.f) : h * (1.f / 3.f);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      zb[q] += xb[q];
+      kb[q] = fmaf(step, xb[q], share * ab[q]);
     }
   }
-  const float hb1[2] = {(hb1a[0] + hb1a[1]) + (hb1a[2] + hb1a[3]),
-                        (hb1b[0] + hb1b[1]) + (hb1b[2] + hb1b[3])};
-  const float p1[2] = {hb1[0] * (1.f - h1[0] * h1[0]), hb1[1] * (1.f - h1[1] * h1[1])};
-  g.b1[lane] += p1[0];
-  g.b1[lane + 32] += p1[1];
-  // dW1[u][i] += p1[u] x[i]; xb[i] = sum_u W1[u][i] p1[u]
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    g.W1t[i * kH + lane] += p1[0] * x6[i];
-    g.W1t[i * kH + lane + 32] += p1[1] * x6[i];
-    zb[i] = warp_sum(fmaf(w.W1t[i * kH + lane], p1[0], w.W1t[i * kH + lane + 32] * p1[1]));
-  }
-  g.W1t[6 * kH + lane] += p1[0] * t;
-  g.W1t[6 * kH + lane + 32] += p1[1] * t;
-  for (int d = 0; d < D; ++d) {
-    const int i = 7 + d;
-    g.W1t[i * kH + lane] += p1[0] * c[d];
-    g.W1t[i * kH + lane + 32] += p1[1] * c[d];
-    cb[d] += warp_sum(fmaf(w.W1t[i * kH + lane], p1[0], w.W1t[i * kH + lane + 32] * p1[1]));
+  for (int q = 0; q < 6; ++q) ab[q] = zb[q];
+}
+
+// Row u of every parameter adjoint, summed over the instance's steps. The
+// embedding is constant along the trajectory, so its terms need only the sum
+// of p1.
+struct ParamSums {
+  f2 w2[kH / 2];
+  float w1[7], w3[6], p1, p2, yb;
+};
+__device__ __forceinline__ void add_step(ParamSums& g, int u, const StepSlot& s) {
+#pragma unroll
+  for (int st = 3; st >= 0; --st) {
+    const float p1 = s.p1[st][u], p2 = s.p2[st][u], h2 = s.h2[st][u];
+    const f2 p22 = pk(p2, p2);
+    const float4* h1 = reinterpret_cast<const float4*>(s.h1[st]);
+#pragma unroll
+    for (int m = 0; m < kH / 4; ++m) {
+      const float4 x = h1[m];
+      g.w2[2 * m] = fma2(pk(x.x, x.y), p22, g.w2[2 * m]);
+      g.w2[2 * m + 1] = fma2(pk(x.z, x.w), p22, g.w2[2 * m + 1]);
+    }
+#pragma unroll
+    for (int i = 0; i < 7; ++i) g.w1[i] = fmaf(p1, s.x[st][i], g.w1[i]);
+#pragma unroll
+    for (int o = 0; o < 6; ++o) g.w3[o] = fmaf(h2, s.yb[st][o], g.w3[o]);
+    g.p1 += p1;
+    g.p2 += p2;
+    if (u < 6) g.yb += s.yb[st][u];
   }
 }
 
-__global__ void __launch_bounds__(32 * kOdeWarps) k_ode_bwd(OdeArgs a) {
-  extern __shared__ __align__(16) float smem[];
+__global__ void __launch_bounds__(kBwdThreads) k_ode_bwd(OdeArgs a) {
+  __shared__ __align__(16) StepSlot s_ring[kRing][kTickSteps];
+  __shared__ float s_p1[kH];
   const OdeLayout L = ode_layout(a.D);
-  const int I = L.I;
-  const SW w = load_weights(a.params, L, smem);
-  float* acc_base = smem + sw_floats(I);
-  const int nacc = acc_floats(I);
-  for (int e = threadIdx.x; e < kOdeWarps * nacc; e += blockDim.x) acc_base[e] = 0.f;
-  __syncthreads();
-  const uint32_t lane = threadIdx.x & 31u;
-  const int warp = threadIdx.x >> 5;
-  const int k = blockIdx.x * kOdeWarps + warp;
-  const Acc g = acc_at(acc_base + warp * nacc, I);
-  if (k < a.n_inst) {
-    const int K = a.n_inst;
-    const int S = a.substeps;
-    float c[kMaxD], cb[kMaxD];
-    for (int d = 0; d < a.D; ++d) {
-      c[d] = a.embed[(size_t)k * a.D + d];
-      cb[d] = 0.f;
+  const int u = threadIdx.x & (kGroup - 1), role = threadIdx.x / kGroup;   // warp-uniform
+  const int k = blockIdx.x;
+  const int n_steps = (a.n_times - 1) * a.substeps;
+  const int ticks = (n_steps + kTickSteps - 1) / kTickSteps + 2;
+  const float* c = a.embed + (size_t)k * a.D;
+  const float* p = a.params;
+  // tick n: groups 0 and 1 recompute the steps of tick n, group 2 walks those
+  // of tick n - 1 and group 3 sums those of tick n - 2. Every group runs the
+  // same number of ticks, one CTA barrier each; step s counts from the end.
+  if (role < kTickSteps) {
+    EvalWeights w;
+    load_eval_weights(w, p, L, c, u);
+    for (int n = 0; n < ticks; ++n) {
+      const int s = n * kTickSteps + role;
+      if (s < n_steps) recompute_step(a, w, n_steps - s, k, u, 1 + role, s_ring[n % kRing][role]);
+      __syncthreads();
     }
+  } else if (role == 2) {
+    AdjointWeights w;
+#pragma unroll
+    for (int m = 0; m < kH / 2; ++m)
+      w.w2[m] = pk(p[L.oW2 + (int64_t)(2 * m) * kH + u], p[L.oW2 + (int64_t)(2 * m + 1) * kH + u]);
+    const int i = (u & 31) >> 2;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int m = 4 * ((u & 3) + 4 * (q >> 1)) + 2 * (q & 1);
+      w.w1[q] = i < 6 ? pk(p[L.oW1 + (int64_t)m * L.I + i], p[L.oW1 + (int64_t)(m + 1) * L.I + i])
+                      : pk(0.f, 0.f);
+    }
+#pragma unroll
+    for (int o = 0; o < 6; ++o) w.w3[o] = p[L.oW3 + o * kH + u];
     float ab[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const int n_steps = (a.n_times - 1) * S;
-    for (int i = n_steps; i >= 0; --i) {
-      if (i % S == 0) {
-        // this output time's pose adjoints enter the state's
-        const int j = i / S;
-        const float* zs = a.states + 6 * ((size_t)i * K + k);
-        const float r[3] = {zs[3], zs[4], zs[5]};
-        const float4 gq = *reinterpret_cast<const float4*>(a.g_quat + 4 * ((size_t)j * K + k));
-        float gr[3];
-        quat_from_rotvec_vjp(r, gq, gr);
-        const float* gt = a.g_trans + 3 * ((size_t)j * K + k);
-        ab[0] += gt[0];
-        ab[1] += gt[1];
-        ab[2] += gt[2];
-        ab[3] += gr[0];
-        ab[4] += gr[1];
-        ab[5] += gr[2];
-      }
-      if (i == 0) break;
-      const int jj = (i - 1) / S, s = (i - 1) - jj * S;
-      const float t0 = a.times[jj];
-      const float h = (a.times[jj + 1] - t0) / (float)S;
-      const float t = t0 + (float)s * h;
-      float z[6];
-      const float* zs = a.states + 6 * ((size_t)(i - 1) * K + k);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) z[q] = zs[q];
-      // the step's four stages again, with their hidden activations
-      float kk[6], u2[6], u3[6], u4[6];
-      float h1a[2], h2a[2], h1b[2], h2b[2], h1c[2], h2c[2], h1d[2], h2d[2];
-      eval_f(w, I, z, t, c, a.D, lane, kk, h1a, h2a);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) u2[q] = fmaf(0.5f * h, kk[q], z[q]);
-      eval_f(w, I, u2, t + 0.5f * h, c, a.D, lane, kk, h1b, h2b);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) u3[q] = fmaf(0.5f * h, kk[q], z[q]);
-      eval_f(w, I, u3, t + 0.5f * h, c, a.D, lane, kk, h1c, h2c);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) u4[q] = fmaf(h, kk[q], z[q]);
-      eval_f(w, I, u4, t + h, c, a.D, lane, kk, h1d, h2d);
-      // z' = z + h/6 (k1 + 2 k2 + 2 k3 + k4), stages in reverse
-      float zb[6], kb[6], xb[6];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        zb[q] = ab[q];
-        kb[q] = h * (1.f / 6.f) * ab[q];
-      }
-      vjp_f(w, g, I, u4, t + h, c, a.D, h1d, h2d, kb, lane, xb, cb);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        zb[q] += xb[q];
-        kb[q] = fmaf(h, xb[q], h * (1.f / 3.f) * ab[q]);
-      }
-      vjp_f(w, g, I, u3, t + 0.5f * h, c, a.D, h1c, h2c, kb, lane, xb, cb);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        zb[q] += xb[q];
-        kb[q] = fmaf(0.5f * h, xb[q], h * (1.f / 3.f) * ab[q]);
-      }
-      vjp_f(w, g, I, u2, t + 0.5f * h, c, a.D, h1b, h2b, kb, lane, xb, cb);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        zb[q] += xb[q];
-        kb[q] = fmaf(0.5f * h, xb[q], h * (1.f / 6.f) * ab[q]);
-      }
-      vjp_f(w, g, I, z, t, c, a.D, h1a, h2a, kb, lane, xb, cb);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) ab[q] = zb[q] + xb[q];
+    for (int n = 0; n < ticks; ++n) {
+      if (n > 0)
+        for (int q = 0; q < kTickSteps; ++q)
+          if ((n - 1) * kTickSteps + q < n_steps) walk_step(w, u, 3, s_ring[(n - 1) % kRing][q], ab);
+      __syncthreads();
     }
-    if (lane == 0) {
-      for (int q = 0; q < 6; ++q) a.g_z0[6 * (size_t)k + q] += ab[q];
-      for (int d = 0; d < a.D; ++d) a.g_embed[(size_t)k * a.D + d] += cb[d];
+    if (u == 0) {
+      float g[6];
+      pose_adjoint(a, 0, k, g);
+#pragma unroll
+      for (int q = 0; q < 6; ++q) a.g_z0[6 * (size_t)k + q] += ab[q] + g[q];
     }
-  }
-  __syncthreads();
-  // the CTA's sums of the warps' accumulators, added to the caller's buffer
-  for (int e = threadIdx.x; e < nacc; e += blockDim.x) {
-    float v = 0.f;
-    for (int q = 0; q < kOdeWarps; ++q) v += acc_base[q * nacc + e];
-    if (v == 0.f) continue;
-    int64_t dst;
-    if (e < I * kH) {                                   // dW1t[i][u] -> W1[u][i]
-      const int i = e / kH, u = e - i * kH;
-      dst = L.oW1 + (int64_t)u * I + i;
-    } else if (e < I * kH + kH) {
-      dst = L.ob1 + (e - I * kH);
-    } else if (e < I * kH + kH + kH * kH) {             // dW2t[j][u] -> W2[u][j]
-      const int r = e - (I * kH + kH);
-      const int j = r / kH, u = r - j * kH;
-      dst = L.oW2 + (int64_t)u * kH + j;
-    } else if (e < I * kH + 2 * kH + kH * kH) {
-      dst = L.ob2 + (e - (I * kH + kH + kH * kH));
-    } else if (e < I * kH + 2 * kH + kH * kH + 6 * kH) {
-      dst = L.oW3 + (e - (I * kH + 2 * kH + kH * kH));
-    } else {
-      dst = L.ob3 + (e - (I * kH + 2 * kH + kH * kH + 6 * kH));
+  } else {
+    ParamSums g = {};
+    for (int n = 0; n < ticks; ++n) {
+      if (n > 1)
+        for (int q = 0; q < kTickSteps; ++q)
+          if ((n - 2) * kTickSteps + q < n_steps) add_step(g, u, s_ring[(n - 2) % kRing][q]);
+      __syncthreads();
     }
-    atomicAdd(a.g_params + dst, v);
+    float* out = a.g_params;
+    float* W1 = out + L.oW1 + (int64_t)u * L.I;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) atomicAdd(W1 + i, g.w1[i]);
+    for (int d = 0; d < a.D; ++d) atomicAdd(W1 + 7 + d, g.p1 * c[d]);
+    atomicAdd(out + L.ob1 + u, g.p1);
+    atomicAdd(out + L.ob2 + u, g.p2);
+#pragma unroll
+    for (int m = 0; m < kH / 2; ++m) {
+      float x, y;
+      upk(g.w2[m], x, y);
+      atomicAdd(out + L.oW2 + (int64_t)u * kH + 2 * m, x);
+      atomicAdd(out + L.oW2 + (int64_t)u * kH + 2 * m + 1, y);
+    }
+#pragma unroll
+    for (int o = 0; o < 6; ++o) atomicAdd(out + L.oW3 + o * kH + u, g.w3[o]);
+    if (u < 6) atomicAdd(out + L.ob3 + u, g.yb);
+    // dL/dc = W1[:, 7:]^T sum p1
+    s_p1[u] = g.p1;
+    group_sync(4);
+    if (u < a.D) {
+      float v = 0.f;
+      for (int m = 0; m < kH; ++m) v = fmaf(p[L.oW1 + (int64_t)m * L.I + 7 + u], s_p1[m], v);
+      a.g_embed[(size_t)k * a.D + u] += v;
+    }
   }
 }
 
@@ -466,10 +503,7 @@ cudaError_t launch_ode_fwd(const s3r_ode_net* net, int n_inst, const float* z0, 
   a.states = states;
   a.quat = quat;
   a.trans = trans;
-  const size_t smem = sizeof(float) * (size_t)sw_floats(7 + a.D);
-  cudaError_t e = cudaFuncSetAttribute(k_ode_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_ode_fwd<<<(n_inst + kOdeWarps - 1) / kOdeWarps, 32 * kOdeWarps, smem, st>>>(a);
+  k_ode_fwd<<<n_inst, kGroup, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -491,11 +525,7 @@ cudaError_t launch_ode_bwd(const s3r_ode_net* net, int n_inst, const float* time
   a.g_params = g_params;
   a.g_embed = g_embed;
   a.g_z0 = g_z0;
-  const int I = 7 + a.D;
-  const size_t smem = sizeof(float) * ((size_t)sw_floats(I) + (size_t)kOdeWarps * acc_floats(I));
-  cudaError_t e = cudaFuncSetAttribute(k_ode_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_ode_bwd<<<(n_inst + kOdeWarps - 1) / kOdeWarps, 32 * kOdeWarps, smem, st>>>(a);
+  k_ode_bwd<<<n_inst, kBwdThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
