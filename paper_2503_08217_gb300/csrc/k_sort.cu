@@ -246,6 +246,7 @@ constexpr int kDupThreads = 256;
 constexpr int kExpItems = S3R_DUP_EXPAND_ITEMS;       // outputs per thread per chunk
 constexpr int kExpChunk = kDupThreads * kExpItems;    // outputs per chunk
 static_assert(kExpChunk >= kDupChunkMin, "the chunk map is sized for chunks of kDupChunkMin");
+static_assert(kExpChunk % 32 == 0, "a chunk clears whole words of contributor bits");
 static_assert(kExpItems <= 14, "above 14 outputs per thread the staged chunk exceeds 48 KB of shared memory");
 
 constexpr float kSpanPad = 0.05f;        // pixels, on the strips and the column bounds
@@ -347,6 +348,9 @@ struct DupArgs {
   int64_t cap_splats, cap_dups;
   uint32_t* ctr;
   unsigned long long* lookback;
+  uint32_t* contrib;       // [bands][contrib_words] the forward's contributor bits, cleared here
+  int64_t contrib_words;
+  int bands;
 };
 
 constexpr int kTilesThreads = 256;
@@ -701,7 +705,6 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
   const int64_t n = min((int64_t)a.ctr[kCtrSplats], a.cap_splats);
   const int64_t total = min((int64_t)a.ctr[kCtrDups], a.cap_dups);
   const int64_t n_chunks = (total + kExpChunk - 1) / kExpChunk;
-  const uint32_t lane = lane_id();
   for (;;) {
     if (threadIdx.x == 0) s_chunk = atomicAdd(a.ctr + kCtrTileBase + kStageExpand, 1u);
     __syncthreads();
@@ -758,7 +761,13 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
       __stcs(a.dup_key + O0 + i, s_key[i]);
       __stcs(a.dup_val + O0 + i, s_val[i]);
     }
-    (void)lane;
+    // the contributor bits of the chunk's pair positions, for the forward: as
+    // many words as there are pairs, where clearing them for the whole pair
+    // capacity in the tile-range launch (a few CTAs on small images) took most
+    // of that launch
+    for (int b = 0; b < a.bands; ++b)
+      for (uint32_t i = threadIdx.x; i < (O1 - O0 + 31u) / 32u; i += kDupThreads)
+        a.contrib[b * a.contrib_words + O0 / 32u + i] = 0u;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < a.tile_passes * kRadix; i += kDupThreads) {
@@ -769,39 +778,39 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
 
 // Tile ranges and the blend queue's classes, one thread per tile: the
 // tile's first pair is the lower bound of its id in the sorted pair keys
-// (binary search), its end the next tile's first pair (the neighbouring lane's
+// (a search), its end the next tile's first pair (the neighbouring lane's
 // search). Every tile's [start, end) is written ([0, 0) for a tile without
 // pairs), and the tile is filed under class clz(end - start) (32 for the
 // empty ones): a shared count per class, one global atomic per class and
-// block for the block's slots, then the ids. The same launch clears the
-// forward's contributor bits.
+// block for the block's slots, then the ids. The launch is bound by the latency
+// of the search's dependent loads, so a step probes seven keys at once and
+// keeps an eighth: 9 steps over 28 million pairs where halving takes 25.
 constexpr int kRangeThreads = 256;
 
+// First position whose key is not below v, among n sorted keys.
 __device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t* __restrict__ keys, uint32_t n,
                                                     uint32_t v) {
-  uint32_t lo = 0, len = n;
-  while (len > 0) {
-    const uint32_t half = len >> 1;
-    if (__ldg(keys + lo + half) < v) {
-      lo += half + 1;
-      len -= half + 1;
-    } else {
-      len = half;
-    }
+  uint32_t lo = 0, len = n;   // the answer is in [lo, lo + len]
+  while (len >= 8) {
+    const uint32_t s = len >> 3;
+    uint32_t below = 0;       // of the seven probes at the eighths' last keys
+#pragma unroll
+    for (uint32_t i = 1; i < 8; ++i) below += __ldg(keys + lo + i * s - 1) < v ? 1u : 0u;
+    lo += below * s;
+    len = below == 7 ? len - 7 * s : s - 1;
   }
-  return lo;
+  uint32_t below = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 7; ++i) below += (i < len && __ldg(keys + lo + i) < v) ? 1u : 0u;
+  return lo + below;
 }
 
 __global__ void __launch_bounds__(kRangeThreads) k_tile_ranges(
     const uint32_t* __restrict__ keys, const uint32_t* ctr, int64_t cap, int tiles,
-    uint2* __restrict__ ranges, uint32_t* class_cnt, uint32_t* __restrict__ class_list,
-    uint32_t* __restrict__ contrib, int64_t contrib_words) {
+    uint2* __restrict__ ranges, uint32_t* class_cnt, uint32_t* __restrict__ class_list) {
   __shared__ uint32_t s_cnt[kTileClasses], s_base[kTileClasses];
   const uint32_t K = (uint32_t)min((int64_t)ctr[kCtrDups], cap);
   const uint32_t lane = lane_id();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < contrib_words;
-       i += (int64_t)gridDim.x * blockDim.x)
-    contrib[i] = 0u;
   for (int base = blockIdx.x * kRangeThreads; base < tiles; base += gridDim.x * kRangeThreads) {
     if (threadIdx.x < kTileClasses) s_cnt[threadIdx.x] = 0u;
     __syncthreads();
@@ -883,6 +892,9 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
   d.lookback = ws->lookback;
   d.hist = ws->hist + kHistTile * kRadix;
   d.tile_passes = ws->tile_passes;
+  d.contrib = ws->contrib;
+  d.contrib_words = ws->contrib_words;
+  d.bands = 2;
   {
     static thread_local int tiles_per_sm = 0;
     if (!tiles_per_sm) tiles_per_sm = per_sm_for((const void*)k_splat_tiles, kTilesThreads);
@@ -931,8 +943,7 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   ws->dup_final = ws->tile_passes & 1;
-  // every tile's range and class (the blend queue), and the cleared
-  // contributor bits of the forward
+  // every tile's range and class (the blend queue)
   {
     const int tiles = ws->views.total_tiles;
     int64_t grid = (tiles + kRangeThreads - 1) / kRangeThreads;
@@ -941,7 +952,7 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     KernelTimer timer(ws, kKTileRanges, st);
     k_tile_ranges<<<(unsigned)grid, kRangeThreads, 0, st>>>(
         ws->dup_key[ws->dup_final], ws->ctr, ws->cap.max_duplicates, tiles, ws->ranges,
-        ws->tile_class_cnt, ws->tile_class_list, ws->contrib, 2 * ws->contrib_words);
+        ws->tile_class_cnt, ws->tile_class_list);
   }
   return cudaGetLastError();
 }
