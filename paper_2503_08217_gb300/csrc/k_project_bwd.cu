@@ -503,14 +503,29 @@ cudaError_t launch_deg(s3r_workspace* ws, const BwdArgs& a, cudaStream_t st) {
   const int nk = ws->n_inst + 1;
   const size_t smem = sizeof(float) * kWarps * ShStage<DEG>::kWords +
                       (size_t)ws->n_views * nk * 12 * sizeof(float) + sizeof(uint32_t) * (nk + 1) + 16;
+  // The dynamic shared-memory limit is a property of the function, shared by all
+  // threads, and the size depends on the scene: it is raised once to the most
+  // the device allows, so that no thread's scene lowers it under another's.
+  static thread_local int most = 0;
   static thread_local size_t cached_smem = 0;
   static thread_local int cached_per_sm = 0;
-  if (smem != cached_smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_project_bwd<DEG>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!most) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_project_bwd<DEG>);
     if (e != cudaSuccess) return e;
+    const int room = optin - (int)fa.sharedSizeBytes;
+    e = cudaFuncSetAttribute(k_project_bwd<DEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+    if (e != cudaSuccess) return e;
+    most = room;
+  }
+  if (smem > (size_t)most) return cudaErrorInvalidValue;
+  if (smem != cached_smem) {
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_project_bwd<DEG>, kThreads, smem);
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_project_bwd<DEG>, kThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     cached_smem = smem;
