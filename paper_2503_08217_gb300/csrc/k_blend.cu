@@ -309,22 +309,18 @@ static_assert(S3R_BLEND_FWD_BLOCKS >= 1 && S3R_BLEND_FWD_BLOCKS * kBandThreads <
 
 struct Band {
   int X0, Y0;              // pixel (0, 0) of this lane
-  float fx[2], fy[kBandRows];
   float bx0, bx1, by0, by1;   // pixel-centre extent of the warp's band
 };
+template <int kWarpsT>
 __device__ __forceinline__ Band band_pixels(const ViewInfo& vi, int lt, int warp, uint32_t lane) {
   Band b;
-  const int bx = (lt % vi.gx) * kTile, by = (lt / vi.gx) * kTile + warp * (kTile / kBandWarps);
+  const int bx = (lt % vi.gx) * kTile, by = (lt / vi.gx) * kTile + warp * (kTile / kWarpsT);
   b.X0 = bx + (int)(lane & 7u);
   b.Y0 = by + (int)(lane >> 3);
-#pragma unroll
-  for (int c = 0; c < 2; ++c) b.fx[c] = (float)(b.X0 + 8 * c) + 0.5f;
-#pragma unroll
-  for (int r = 0; r < kBandRows; ++r) b.fy[r] = (float)(b.Y0 + 4 * r) + 0.5f;
   b.bx0 = bx + 0.5f;
   b.bx1 = bx + 15.5f;
   b.by0 = by + 0.5f;
-  b.by1 = by + (kTile / kBandWarps) - 0.5f;
+  b.by1 = by + (kTile / kWarpsT) - 0.5f;
   return b;
 }
 
@@ -396,31 +392,33 @@ __device__ __forceinline__ float blend_alpha(float p, float al, float nT, int po
   return ab;
 }
 
-// One splat of the forward's walk over a warp's four pixels per lane (two
-// packed pairs). kClamp: the splat's opacity exceeds 0.99, so alpha = o G may
+// One splat of the forward's walk over a lane's pixels, kPairs packed pairs:
+// two columns of two rows each with two warps per tile, one row of two columns
+// with four (FX and FY hold the pairs' pixel centres accordingly). kClamp: the splat's opacity exceeds 0.99, so alpha = o G may
 // reach the 0.99 cap; for o <= 0.99 it cannot (G = 2^p <= 1 where p <= 0, up
 // to the last ulp of ex2.approx at p = 0), and the clamp is left out. The
 // backward takes the same branch per splat, and the FP64 o G of the exact
 // definition never reaches the cap for those splats either.
-template <bool kCount, bool kClamp>
+template <bool kCount, bool kClamp, int kPairs>
 __device__ __forceinline__ void fwd_splat(const float4 q0, const float4 q1, const float4 q2,
                                           const float4 q3, const float2 qu, const f2 FY,
-                                          const f2 (&FX)[2], const f2 ONE, int pos, f2 (&T2)[2],
-                                          f2 (&C2)[2][3], int (&last)[kBandPix],
-                                          int (&endp)[kBandPix], float (&floor_)[kBandPix],
-                                          uint32_t& n_eval, bool& any_blend) {
+                                          const f2 (&FX)[kPairs], const f2 ONE, int pos,
+                                          f2 (&T2)[kPairs], f2 (&C2)[kPairs][3],
+                                          int (&last)[2 * kPairs], int (&endp)[2 * kPairs],
+                                          float (&floor_)[2 * kPairs], uint32_t& n_eval,
+                                          bool& any_blend) {
   // a blended pixel takes alpha >= 1/255 > 0, a skipped one 0: the splat was
   // blended somewhere in the lane's pixels iff the applied alphas sum above 0
   f2 ab_sum;
   const f2 A2 = pk(q0.x, q0.y), B2 = pk(q0.z, q0.w), C2c = pk(q1.x, q1.y), O2 = pk(q1.z, q1.w);
   const f2 R2 = pk(q2.x, q2.y), G2 = pk(q2.z, q2.w), Bl2 = pk(q3.x, q3.y), V2 = pk(q3.z, q3.w);
   const f2 U2 = pk(qu.x, qu.y);
-  // the rows' dy and the dy terms of the exponent, shared by both columns
+  // the rows' dy and the dy terms of the exponent, shared by the pairs
   const f2 dy = sub2(V2, FY);
   const f2 bdy = mul2(B2, dy);
   const f2 cdy = mul2(mul2(C2c, dy), dy);
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
+  for (int c = 0; c < kPairs; ++c) {
     const f2 dx = sub2(U2, FX[c]);
     const f2 pw = fma2(dx, fma2(A2, dx, bdy), cdy);
     float p[2], raw[2];
@@ -433,7 +431,7 @@ __device__ __forceinline__ void fwd_splat(const float4 q0, const float4 q1, cons
     upk(mul2(T2[c], sub2(ONE, pk(al[0], al[1]))), nT[0], nT[1]);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      const int k = c * kBandRows + r;
+      const int k = 2 * c + r;
       const bool was_done = floor_[k] > 1.f;
       if constexpr (kCount) n_eval += was_done ? 0u : 1u;
       // one select: T (1 - 0) = T exactly where the splat is not blended
@@ -453,19 +451,31 @@ __device__ __forceinline__ void fwd_splat(const float4 q0, const float4 q1, cons
   any_blend = s0 + s1 > 0.f;
 }
 
-__device__ __forceinline__ bool all_stopped(const float (&floor_)[kBandPix]) {
-  static_assert(kBandPix == 4, "four pixels per lane");
-  return fminf(fminf(floor_[0], floor_[1]), fminf(floor_[2], floor_[3])) > 1.f;
+template <int kPix>
+__device__ __forceinline__ bool all_stopped(const float (&floor_)[kPix]) {
+  float least = floor_[0];
+#pragma unroll
+  for (int k = 1; k < kPix; ++k) least = fminf(least, floor_[k]);
+  return least > 1.f;
 }
 
 // S3R_BLEND_FWD_BLOCKS: 18 blocks per SM (56 registers). At the surround rig
 // (27.7M pairs, 1.07G evaluated) 18 blocks took 1.043 ms, 20 (48 registers)
 // 1.084 ms and 16 (64 registers) 1.148 ms: the kernel needs the warps, and a
 // few registers more than 48 end the spills.
-template <bool kCount>
-__global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fwd(const __grid_constant__ ViewSet vs,
-                                                            BlendArgs a) {
-  static_assert(kBandRows == 2, "the packed forward pairs the two rows of a lane's column");
+//
+// kWarpsT: warps per tile. Two (16x8 bands, four pixels per lane) share a
+// splat's loads and loop between the most pixels. Where the image has so few
+// tiles that all of them are resident at once, the time is that of the longest
+// list walked by one pair of warps, and four (16x4 bands, two pixels per lane)
+// walk it faster: see launch_render_fwd for the line and both sides' times. The
+// contributor bits stay those of the backward's 16x8 bands, two warps adding
+// to each.
+template <bool kCount, int kWarpsT>
+__global__ void __launch_bounds__(32 * kWarpsT, S3R_BLEND_FWD_BLOCKS * kBandWarps / kWarpsT) k_blend_fwd(
+    const __grid_constant__ ViewSet vs, BlendArgs a) {
+  static_assert(kWarpsT == 2 || kWarpsT == 4, "bands of 16x8 or 16x4 pixels");
+  constexpr int kPairs = 4 / kWarpsT, kPix = 2 * kPairs, kThreadsT = 32 * kWarpsT;
   __shared__ float4 s_p0[kBatchFwd];   // A2 A2 B2 B2
   __shared__ float4 s_p1[kBatchFwd];   // C2 C2 o o
   __shared__ float4 s_p2[kBatchFwd];   // r r g g
@@ -489,36 +499,44 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
     const int lt = tile - vi.tile_base;
     const int warp = threadIdx.x >> 5;
     const uint32_t lane = lane_id();
-    const Band P = band_pixels(vi, lt, warp, lane);
+    const Band P = band_pixels<kWarpsT>(vi, lt, warp, lane);
+    // pixel k = 2 c + r of the lane: column c, row r of two warps' bands, else
+    // column r of the one row
+    int px[kPix], py[kPix];
+#pragma unroll
+    for (int k = 0; k < kPix; ++k) {
+      px[k] = P.X0 + 8 * (kPairs == 2 ? k >> 1 : k);
+      py[k] = P.Y0 + (kPairs == 2 ? 4 * (k & 1) : 0);
+    }
     const uint2 range = a.ranges[tile];
     const int n = (int)(range.y - range.x);
-    const f2 FY = pk(P.fy[0], P.fy[1]);
-    const f2 FX[2] = {pk(P.fx[0], P.fx[0]), pk(P.fx[1], P.fx[1])};
+    const f2 FY = pk((float)py[0] + 0.5f, (float)py[1] + 0.5f);
+    f2 FX[kPairs];
     const f2 ONE = pk(1.f, 1.f);
 
-    // per column c: the pair (row 0, row 1); scalar per-pixel state k = 2c + r
-    f2 T2[2], C2[2][3];
-    int last[kBandPix], endp[kBandPix];
-    float floor_[kBandPix];   // least alpha taken; infinity once the pixel has stopped
+    // per pair; scalar per-pixel state
+    f2 T2[kPairs], C2[kPairs][3];
+    int last[kPix], endp[kPix];
+    float floor_[kPix];   // least alpha taken; infinity once the pixel has stopped
     uint32_t n_eval = 0;
   #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < kPairs; ++c) {
+      FX[c] = pk((float)px[2 * c] + 0.5f, (float)px[2 * c + 1] + 0.5f);
       T2[c] = ONE;
       C2[c][0] = C2[c][1] = C2[c][2] = pk(0.f, 0.f);
-  #pragma unroll
-      for (int r = 0; r < kBandRows; ++r) {
-        const int k = c * kBandRows + r;
-        last[k] = 0;
-        const bool inside = P.X0 + 8 * c < vi.width && P.Y0 + 4 * r < vi.height;
-        floor_[k] = inside ? kAlphaMin : INFINITY;
-        endp[k] = inside ? n : 0;      // positions walked
-      }
     }
-    uint32_t* wbits = a.contrib + warp * a.contrib_words;
+  #pragma unroll
+    for (int k = 0; k < kPix; ++k) {
+      const bool inside = px[k] < vi.width && py[k] < vi.height;
+      last[k] = 0;
+      floor_[k] = inside ? kAlphaMin : INFINITY;
+      endp[k] = inside ? n : 0;      // positions walked
+    }
+    uint32_t* wbits = a.contrib + (warp * kBandWarps / kWarpsT) * a.contrib_words;
     for (int b0 = 0; b0 < n; b0 += kBatchFwd) {
       // whether every pixel has stopped: tested once per chunk and batch, not per splat
       if (__syncthreads_and(all_stopped(floor_))) break;
-      for (int i = threadIdx.x; i < kBatchFwd && b0 + i < n; i += kBandThreads) {
+      for (int i = threadIdx.x; i < kBatchFwd && b0 + i < n; i += kThreadsT) {
         const uint32_t s = a.sorted_splats[range.x + b0 + i];
         const uint4 t0 = a.sp_tin[2 * (size_t)s], t1 = a.sp_tin[2 * (size_t)s + 1];
         const float2 xy = make_float2(__uint_as_float(t0.x), __uint_as_float(t0.y));
@@ -559,10 +577,10 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
           bool any_blend = false;
           // warp-uniform: every lane walks the same splat
           if (q1.z > kAlphaMax)
-            fwd_splat<kCount, true>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, floor_,
+            fwd_splat<kCount, true, kPairs>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, floor_,
                                     n_eval, any_blend);
           else
-            fwd_splat<kCount, false>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, floor_,
+            fwd_splat<kCount, false, kPairs>(q0, q1, q2, q3, qu, FY, FX, ONE, pos, T2, C2, last, endp, floor_,
                                      n_eval, any_blend);
           if (__any_sync(0xffffffffu, any_blend)) blended |= 1u << (j - c0);
         }
@@ -573,7 +591,7 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
       // work accounting, one 64-bit atomic per warp and counter
       unsigned long long walked = 0;
   #pragma unroll
-      for (int k = 0; k < kBandPix; ++k) walked += (unsigned long long)endp[k];
+      for (int k = 0; k < kPix; ++k) walked += (unsigned long long)endp[k];
       unsigned long long evald = n_eval;
   #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -585,18 +603,17 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_FWD_BLOCKS) k_blend_fw
     }
     const int64_t plane = (int64_t)vi.width * vi.height;
   #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < kPairs; ++c) {
       float T[2], Cr[2], Cg[2], Cb[2];
       upk(T2[c], T[0], T[1]);
       upk(C2[c][0], Cr[0], Cr[1]);
       upk(C2[c][1], Cg[0], Cg[1]);
       upk(C2[c][2], Cb[0], Cb[1]);
   #pragma unroll
-      for (int r = 0; r < kBandRows; ++r) {
-        const int k = c * kBandRows + r;
-        const int px = P.X0 + 8 * c, py = P.Y0 + 4 * r;
-        if (px < vi.width && py < vi.height) {
-          const int64_t pix = (int64_t)py * vi.width + px;
+      for (int r = 0; r < 2; ++r) {
+        const int k = 2 * c + r;
+        if (px[k] < vi.width && py[k] < vi.height) {
+          const int64_t pix = (int64_t)py[k] * vi.width + px[k];
           float* o = a.out + 3 * (int64_t)vi.pix_base + pix;
           o[0] = fmaf(T[r], a.bg[0], Cr[r]);
           o[plane] = fmaf(T[r], a.bg[1], Cg[r]);
@@ -1046,17 +1063,25 @@ static BlendArgs make_args(s3r_workspace* ws) {
   return a;
 }
 
-// Resident CTAs per SM of a blend instantiation, queried once per process.
+// Resident CTAs per SM of a blend instantiation, queried once per thread.
 template <typename K>
-int blend_blocks_per_sm(K kernel, int* cache) {
+int blend_blocks_per_sm(K kernel, int threads, int* cache) {
   if (*cache == 0) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBandThreads, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
     *cache = per_sm;
   }
   return *cache;
+}
+
+template <bool kCount, int kWarpsT>
+void launch_fwd(s3r_workspace* ws, const BlendArgs& a, cudaStream_t st) {
+  static thread_local int per_sm = 0;
+  constexpr int kThreadsT = 32 * kWarpsT;
+  const int g = ws->num_sms * blend_blocks_per_sm(k_blend_fwd<kCount, kWarpsT>, kThreadsT, &per_sm);
+  k_blend_fwd<kCount, kWarpsT><<<g, kThreadsT, 0, st>>>(ws->views, a);
 }
 
 cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cudaStream_t st) {
@@ -1070,14 +1095,15 @@ cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cu
     if ((e = cudaMemsetAsync(a.pairs, 0, 2 * sizeof(unsigned long long), st)) != cudaSuccess) return e;
   }
   // the contributor bits were cleared by the sort's pair expansion
-  static thread_local int per_sm[2] = {0, 0};
+  // four warps per tile where every tile is resident at once with two (see k_blend_fwd)
+  const bool few = ws->views.total_tiles <= ws->num_sms * S3R_BLEND_FWD_BLOCKS;
   KernelTimer timer(ws, kKBlendFwd, st);
   if (ws->counting) {
-    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_fwd<true>, &per_sm[1]);
-    k_blend_fwd<true><<<g, kBandThreads, 0, st>>>(ws->views, a);
+    if (few) launch_fwd<true, 4>(ws, a, st);
+    else launch_fwd<true, 2>(ws, a, st);
   } else {
-    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_fwd<false>, &per_sm[0]);
-    k_blend_fwd<false><<<g, kBandThreads, 0, st>>>(ws->views, a);
+    if (few) launch_fwd<false, 4>(ws, a, st);
+    else launch_fwd<false, 2>(ws, a, st);
   }
   ws->sp_grad_clean = 1;
   return cudaGetLastError();
@@ -1111,10 +1137,10 @@ cudaError_t launch_render_bwd(s3r_workspace* ws, const float* bg, const float* d
   static thread_local int per_sm[2] = {0, 0};
   KernelTimer timer(ws, kKBlendBwd, st);
   if (ws->counting) {
-    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_bwd<true>, &per_sm[1]);
+    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_bwd<true>, kBandThreads, &per_sm[1]);
     k_blend_bwd<true><<<g, kBandThreads, 0, st>>>(ws->views, a);
   } else {
-    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_bwd<false>, &per_sm[0]);
+    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_bwd<false>, kBandThreads, &per_sm[0]);
     k_blend_bwd<false><<<g, kBandThreads, 0, st>>>(ws->views, a);
   }
   return cudaGetLastError();

@@ -24,18 +24,27 @@ constexpr int kWarpSpan = kRounds * 32 * 2;           // Gaussians per warp
 constexpr int kTileSpan = kWarps * kWarpSpan;         // 4096 Gaussians per tile
 constexpr int kChunkTiles = kThreads / kWarps;        // tiles a CTA holds (one offset per thread)
 
-// W_v * P_k for every segment k of view v (k = 0: identity pose), and the
-// camera centre in the segment's frame, computed in FP64 once per call; the
-// block's threads stride over the segments.
-__device__ __forceinline__ void compose_view(const ViewSet& vs, int v,
+// W_v * P_k for segments k of view v (k = 0: identity pose), and the camera
+// centre in the segment's frame, computed in FP64 once per call: item m is the
+// (m / per_view)-th view's segments 32 (m % per_view) .. + 31, one per lane of
+// the CTA's first warp. FP64 issues at a sixteenth of a warp per cycle here, so
+// an SM's time is that of its FP64 instructions: an item is one warp's worth,
+// and the inverse takes one division.
+constexpr int kComposeSegs = 32;
+__host__ __device__ inline int compose_items(int n_views, int n_inst) {
+  return n_views * ((n_inst + kComposeSegs) / kComposeSegs);
+}
+__device__ __forceinline__ void compose_item(const ViewSet& vs, int m,
                                              const float4* __restrict__ pose_q,
                                              const float* __restrict__ pose_t, int n_inst,
                                              InstMat* __restrict__ out) {
-  const int nk = n_inst + 1;
+  const int nk = n_inst + 1, per_view = (nk + kComposeSegs - 1) / kComposeSegs;
+  const int v = m / per_view;
   const float* Vf = vs.v[v].V;
   double V[12];
   for (int i = 0; i < 12; ++i) V[i] = Vf[i];
-  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+  const int k = (m - v * per_view) * kComposeSegs + (int)threadIdx.x;
+  if (threadIdx.x < kComposeSegs && k < nk) {
     double R[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1}, t[3] = {0, 0, 0};
     if (k > 0) {
       const float4 qf = pose_q[k - 1];
@@ -57,9 +66,10 @@ __device__ __forceinline__ void compose_view(const ViewSet& vs, int v,
     const double c00 = A[4] * A[8] - A[5] * A[7], c01 = A[5] * A[6] - A[3] * A[8],
                  c02 = A[3] * A[7] - A[4] * A[6];
     const double det = A[0] * c00 + A[1] * c01 + A[2] * c02;
-    const double Ai[9] = {c00 / det, (A[2] * A[7] - A[1] * A[8]) / det, (A[1] * A[5] - A[2] * A[4]) / det,
-                          c01 / det, (A[0] * A[8] - A[2] * A[6]) / det, (A[2] * A[3] - A[0] * A[5]) / det,
-                          c02 / det, (A[1] * A[6] - A[0] * A[7]) / det, (A[0] * A[4] - A[1] * A[3]) / det};
+    const double id = 1.0 / det;
+    const double Ai[9] = {c00 * id, (A[2] * A[7] - A[1] * A[8]) * id, (A[1] * A[5] - A[2] * A[4]) * id,
+                          c01 * id, (A[0] * A[8] - A[2] * A[6]) * id, (A[2] * A[3] - A[0] * A[5]) * id,
+                          c02 * id, (A[1] * A[6] - A[0] * A[7]) * id, (A[0] * A[4] - A[1] * A[3]) * id};
     InstMat m;
     for (int r = 0; r < 3; ++r) {
       for (int c = 0; c < 3; ++c) m.m[4 * r + c] = (float)A[3 * r + c];
@@ -93,7 +103,8 @@ __device__ __forceinline__ uint32_t interleave16(uint32_t even, uint32_t odd) {
 
 // The first launch of a call sequence also does the call's set-up, so that
 // it needs no launch of its own: its first CTAs compose the instance
-// matrices of the views (for the projection that follows), and the last CTA
+// matrices of the views (for the projection that follows; they do nothing else
+// where the grid has room for them besides a CTA per chunk), and the last CTA
 // to finish zeroes the per-call counters, histograms and tile-class counts,
 // bumps the call counter (epoch) and resets the compaction's tile counter.
 // The compaction's look-back words carry the tag of the new epoch, read by
@@ -107,6 +118,10 @@ struct CallSetup {
   uint32_t* hist;                    // null: no histograms
   uint32_t* tile_class_cnt;          // null: no tile classes
   int64_t lookback_words;
+  int compose_only;                  // CTAs at the start of the grid that only compose
+  uint32_t* out_count;               // not null (the selection without a workspace): where
+                                     // the last CTA writes the list's length, or
+                                     // S3R_STATIC_TIMEOUT, and clears the status
 };
 
 __device__ void call_setup_last(uint32_t* ctr, unsigned long long* lookback, const CallSetup& c,
@@ -124,6 +139,11 @@ __device__ void call_setup_last(uint32_t* ctr, unsigned long long* lookback, con
   if (threadIdx.x == 0) {
     ctr[kCtrEpoch] = epoch;
     if (n_tiles == 0) ctr[kCtrSelected] = 0;
+    if (c.out_count) {
+      *c.out_count = (__ldcg(ctr + kCtrStatus) & kStatusTimeout) ? S3R_STATIC_TIMEOUT
+                                                        : (n_tiles ? __ldcg(ctr + kCtrSelected) : 0u);
+      ctr[kCtrStatus] = 0;
+    }
   }
   // look-back tags keep the epoch's low 26 bits: before the call whose tags
   // wrap around, every word is cleared (once per 67,108,864 calls)
@@ -155,8 +175,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_compact(const __grid_constant__
   __shared__ uint32_t s_tmp[kWarps];
   __shared__ uint32_t s_chunk;
   __shared__ bool s_last;
-  for (int v = blockIdx.x; v < setup.n_views; v += gridDim.x)
-    compose_view(vs, v, setup.pose_q, setup.pose_t, setup.n_inst, setup.mats);
+  if (setup.n_views > 0) {
+    const int items = compose_items(setup.n_views, setup.n_inst);
+    for (int m = blockIdx.x; m < items; m += gridDim.x)
+      compose_item(vs, m, setup.pose_q, setup.pose_t, setup.n_inst, setup.mats);
+  }
   const int warp = threadIdx.x >> 5;
   const uint32_t lane = lane_id();
   const uint32_t tag = stage_tag(ctr[kCtrEpoch] + 1u, kStageCompact);
@@ -179,7 +202,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_compact(const __grid_constant__
       }
     }
   };
-  for (;;) {
+  // where the CTAs that stream are as many as the chunks, each takes one
+  const bool one_chunk = n_chunks <= (int64_t)gridDim.x - setup.compose_only;
+  while ((int)blockIdx.x >= setup.compose_only) {
     if (threadIdx.x == 0) s_chunk = atomicAdd(ctr + kCtrTileBase + kStageCompact, 1u);
     __syncthreads();
     const int64_t chunk = s_chunk;
@@ -259,6 +284,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_compact(const __grid_constant__
         out += __popc(b0) + __popc(b1);
       }
     }
+    if (one_chunk) break;
     __syncthreads();   // s_chunk / s_bits / s_off reuse
   }
   // the last CTA to finish does the call's set-up for the launches after it
@@ -279,8 +305,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_compact(const __grid_constant__
 struct CompactGrid {
   int per;
   unsigned grid;
+  int compose_only;
 };
-CompactGrid compact_grid(int64_t n, int sms) {
+CompactGrid compact_grid(int64_t n, int sms, int items) {
   // occupancy is queried once (outside any graph capture: the first call)
   static int per_sm = 0;
   if (!per_sm) {
@@ -297,7 +324,8 @@ CompactGrid compact_grid(int64_t n, int sms) {
   const int64_t n_chunks = (n_tiles + per - 1) / per;
   int64_t grid = n_chunks < resident ? n_chunks : resident;
   if (grid < 1) grid = 1;
-  return {(int)per, (unsigned)grid};
+  const bool room = grid + items <= resident;
+  return {(int)per, (unsigned)(grid + (room ? items : 0)), room ? items : 0};
 }
 
 }  // namespace
@@ -305,7 +333,7 @@ CompactGrid compact_grid(int64_t n, int sms) {
 cudaError_t launch_compact(s3r_workspace* ws, const s3r_scene* sc, const s3r_poses* poses,
                            const float* vis, float t, cudaStream_t st) {
   const int64_t n = sc->n;
-  const CompactGrid cg = compact_grid(n, ws->num_sms);
+  const CompactGrid cg = compact_grid(n, ws->num_sms, compose_items(ws->n_views, sc->n_inst));
   CallSetup c;
   c.n_views = ws->n_views;
   c.pose_q = reinterpret_cast<const float4*>(poses ? poses->quat : nullptr);
@@ -315,6 +343,8 @@ cudaError_t launch_compact(s3r_workspace* ws, const s3r_scene* sc, const s3r_pos
   c.hist = ws->hist;
   c.tile_class_cnt = ws->tile_class_cnt;
   c.lookback_words = ws->lookback_words;
+  c.compose_only = cg.compose_only;
+  c.out_count = nullptr;
   KernelTimer timer(ws, kKCompact, st);
   k_compact<<<cg.grid, kThreads, 0, st>>>(ws->views, vis, n, t, cg.per, ws->selected, ws->ctr,
                                           ws->lookback, ws->kept_bits, c);
@@ -377,13 +407,6 @@ s3r_status static_scratch(StaticScratch** out, int* sms) {
   return S3R_OK;
 }
 
-// The list length, or 0xffffffff where a look-back wait of the call gave up
-// (the list is then not valid): the status word is only in the scratch, so
-// the call reports it through its output.
-__global__ void k_static_finish(const uint32_t* ctr, uint32_t* out_count) {
-  *out_count = (ctr[kCtrStatus] & kStatusTimeout) ? 0xffffffffu : ctr[kCtrSelected];
-}
-
 }  // namespace
 }  // namespace s3r
 
@@ -406,21 +429,16 @@ extern "C" s3r_status s3r_select_visible_static(int64_t n, float t, const float*
   s3r_status st = static_scratch(&sc, &sms);
   if (st != S3R_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t n_tiles = (n + kTileSpan - 1) / kTileSpan;
-  // the array keeps the previous call's contents: clear the counters and the
-  // look-back words this call will use
-  cudaError_t e = cudaMemsetAsync(sc->ctr, 0, sizeof(sc->ctr), s);
-  if (e == cudaSuccess && n_tiles > 0)
-    e = cudaMemsetAsync(sc->lookback, 0, sizeof(unsigned long long) * (size_t)n_tiles, s);
+  // The array keeps the previous call's contents: the counters past the epoch
+  // are cleared, the look-back words carry the epoch, which the last CTA
+  // advances, and that CTA also writes the count and clears the status. (Two
+  // clears and a launch for the count besides took 4 us of a small call.)
+  cudaError_t e = cudaMemsetAsync(sc->ctr + kCtrEpoch + 1, 0, sizeof(uint32_t) * (kCtrCount - kCtrEpoch - 1), s);
   if (e == cudaSuccess) {
-    const CompactGrid cg = compact_grid(n, sms);
-    CallSetup none = {0, nullptr, nullptr, 0, nullptr, nullptr, nullptr, 0};
+    const CompactGrid cg = compact_grid(n, sms, 0);
+    CallSetup setup = {0, nullptr, nullptr, 0, nullptr, nullptr, nullptr, kStaticTiles, 0, out_count};
     k_compact<<<cg.grid, kThreads, 0, s>>>(g_no_views, vis_window, n, t, cg.per, out_idx, sc->ctr,
-                                            sc->lookback, nullptr, none);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    k_static_finish<<<1, 1, 0, s>>>(sc->ctr, out_count);
+                                            sc->lookback, nullptr, setup);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return set_last_error(S3R_ERR_CUDA, cudaGetErrorString(e));

@@ -2,30 +2,80 @@
 //   RECORD   Eq. 5: l_s = min(l_s, t), l_e = max(l_e, t) where M_t[i];
 //   FINALIZE Eq. 6: v = (l_s - 0.1, l_e + 0.1), in FP32;
 //   RESET    v = (-1, 1), l = (1, -1): visible at all times, empty life.
-// A plain streaming pass, one Gaussian (one 8-byte pair per array) per
-// thread, so that sub-ranges starting at any index can be passed.
+// A plain streaming pass. Where both arrays are 16-byte aligned a thread takes
+// four pairs of Gaussians (one 128-bit access per pair and array, the four
+// loads issued together); a sub-range that starts at an odd index has only
+// 8-byte alignment and takes one Gaussian per access.
 #include "s3r_internal.cuh"
 
 namespace s3r {
 namespace {
 
-__global__ void k_vis(int64_t n, float t, const uint32_t* __restrict__ mask, float2* life,
-                      float2* vis, int mode) {
+template <int MODE>
+__device__ __forceinline__ void vis_one(int64_t i, float t, uint32_t seen, float2* life, float2* vis) {
+  if (MODE == S3R_VIS_RESET) {
+    vis[i] = make_float2(-1.f, 1.f);
+    life[i] = make_float2(1.f, -1.f);
+  } else if (MODE == S3R_VIS_FINALIZE) {
+    const float2 l = life[i];
+    vis[i] = make_float2(l.x - 0.1f, l.y + 0.1f);
+  } else if (seen & 1u) {
+    const float2 l = life[i];
+    life[i] = make_float2(fminf(l.x, t), fmaxf(l.y, t));
+  }
+}
+
+template <int MODE>
+__global__ void k_vis(int64_t n, float t, const uint32_t* __restrict__ mask, float2* life, float2* vis) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (mode == S3R_VIS_RESET) {
-      vis[i] = make_float2(-1.f, 1.f);
-      life[i] = make_float2(1.f, -1.f);
-    } else if (mode == S3R_VIS_FINALIZE) {
-      const float2 l = life[i];
-      vis[i] = make_float2(l.x - 0.1f, l.y + 0.1f);
-    } else if ((mask[i >> 5] >> (i & 31)) & 1u) {
-      float2 l = life[i];
-      l.x = fminf(l.x, t);
-      l.y = fmaxf(l.y, t);
-      life[i] = l;
+       i += (int64_t)gridDim.x * blockDim.x)
+    vis_one<MODE>(i, t, MODE == S3R_VIS_RECORD ? mask[i >> 5] >> (i & 31) : 0u, life, vis);
+}
+
+constexpr int kVisThreads = 256, kVisPairs = 4;   // pairs of Gaussians per thread
+template <int MODE>
+__global__ void __launch_bounds__(kVisThreads) k_vis_pairs(int64_t n, float t,
+                                                           const uint32_t* __restrict__ mask,
+                                                           float4* life, float4* vis) {
+  const int64_t pairs = n >> 1;
+  const int64_t p0 = (int64_t)blockIdx.x * (kVisThreads * kVisPairs) + threadIdx.x;
+  uint32_t seen[kVisPairs];
+  float4 l[kVisPairs];
+#pragma unroll
+  for (int q = 0; q < kVisPairs; ++q) {
+    const int64_t p = p0 + q * kVisThreads;
+    seen[q] = 3u;
+    if (MODE == S3R_VIS_RECORD) seen[q] = p < pairs ? (mask[p >> 4] >> ((p & 15) * 2)) & 3u : 0u;
+  }
+#pragma unroll
+  for (int q = 0; q < kVisPairs; ++q) {
+    const int64_t p = p0 + q * kVisThreads;
+    if (MODE != S3R_VIS_RESET && p < pairs && seen[q]) l[q] = life[p];
+  }
+#pragma unroll
+  for (int q = 0; q < kVisPairs; ++q) {
+    const int64_t p = p0 + q * kVisThreads;
+    if (p >= pairs || !seen[q]) continue;
+    if (MODE == S3R_VIS_RESET) {
+      vis[p] = make_float4(-1.f, 1.f, -1.f, 1.f);
+      life[p] = make_float4(1.f, -1.f, 1.f, -1.f);
+    } else if (MODE == S3R_VIS_FINALIZE) {
+      vis[p] = make_float4(l[q].x - 0.1f, l[q].y + 0.1f, l[q].z - 0.1f, l[q].w + 0.1f);
+    } else {
+      if (seen[q] & 1u) {
+        l[q].x = fminf(l[q].x, t);
+        l[q].y = fmaxf(l[q].y, t);
+      }
+      if (seen[q] & 2u) {
+        l[q].z = fminf(l[q].z, t);
+        l[q].w = fmaxf(l[q].w, t);
+      }
+      life[p] = l[q];
     }
   }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)   // the last Gaussian of an odd count
+    vis_one<MODE>(n - 1, t, MODE == S3R_VIS_RECORD ? mask[(n - 1) >> 5] >> ((n - 1) & 31) : 0u,
+                  reinterpret_cast<float2*>(life), reinterpret_cast<float2*>(vis));
 }
 
 // Mean absolute error and its gradient; one block-reduced atomic per CTA.
@@ -170,13 +220,31 @@ cudaError_t launch_l1_loss(int64_t n, const float* pred, const float* target, fl
   return cudaGetLastError();
 }
 
+namespace {
+template <int MODE>
+void vis_launch(int64_t n, float t, const uint32_t* mask, float* life, float* vis, cudaStream_t st) {
+  const bool aligned = ((reinterpret_cast<uintptr_t>(life) | reinterpret_cast<uintptr_t>(vis)) & 15u) == 0;
+  const int64_t pair_blocks = (n / 2 + kVisThreads * kVisPairs - 1) / (kVisThreads * kVisPairs);
+  if (aligned && pair_blocks <= 0x7fffffffLL) {
+    k_vis_pairs<MODE><<<(unsigned)(pair_blocks > 0 ? pair_blocks : 1), kVisThreads, 0, st>>>(
+        n, t, mask, reinterpret_cast<float4*>(life), reinterpret_cast<float4*>(vis));
+    return;
+  }
+  int64_t blocks = (n + 255) / 256;
+  if (blocks > (int64_t)sm_count() * 64) blocks = (int64_t)sm_count() * 64;
+  k_vis<MODE><<<(unsigned)blocks, 256, 0, st>>>(n, t, mask, reinterpret_cast<float2*>(life),
+                                                reinterpret_cast<float2*>(vis));
+}
+}  // namespace
+
 cudaError_t launch_visibility(int64_t n, float t, const uint32_t* mask, float* life, float* vis,
                               int mode, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > (int64_t)sm_count() * 64) blocks = (int64_t)sm_count() * 64;
-  k_vis<<<(unsigned)blocks, 256, 0, st>>>(n, t, mask, reinterpret_cast<float2*>(life),
-                                          reinterpret_cast<float2*>(vis), mode);
+  switch (mode) {
+    case S3R_VIS_RESET: vis_launch<S3R_VIS_RESET>(n, t, mask, life, vis, st); break;
+    case S3R_VIS_FINALIZE: vis_launch<S3R_VIS_FINALIZE>(n, t, mask, life, vis, st); break;
+    default: vis_launch<S3R_VIS_RECORD>(n, t, mask, life, vis, st); break;
+  }
   return cudaGetLastError();
 }
 
