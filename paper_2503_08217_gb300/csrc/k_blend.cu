@@ -562,6 +562,7 @@ __device__ __forceinline__ bool all_stopped(const float (&floor_)[kPix]) {
 template <bool kCount, int kWarpsT>
 __global__ void __launch_bounds__(32 * kWarpsT, S3R_BLEND_FWD_BLOCKS * kBandWarps / kWarpsT) k_blend_fwd(
     const __grid_constant__ ViewSet vs, BlendArgs a) {
+  sequence_begin();
   static_assert(kWarpsT == 2 || kWarpsT == 4, "bands of 16x8 or 16x4 pixels");
   constexpr int kPairs = 4 / kWarpsT, kPix = 2 * kPairs, kThreadsT = 32 * kWarpsT;
   constexpr int kAhead = 2;   // splats evaluated together by four warps (1: 0.184 ms, 2: 0.149, 3 and 4: 0.162)
@@ -980,6 +981,7 @@ __device__ __forceinline__ void sum_rows(const float* half_row, const float* nin
 template <bool kCount>
 __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bwd(
     const __grid_constant__ ViewSet vs, BlendArgs a) {
+  sequence_begin();
   static_assert(kBandRows == 2, "the packed backward pairs the two rows of a lane's column");
   constexpr int kT = kBandThreads;
   constexpr int kRows = kBandRows;
@@ -1162,6 +1164,7 @@ __global__ void __launch_bounds__(kBandThreads, S3R_BLEND_BWD_BLOCKS) k_blend_bw
 
 // Zero the per-splat adjoints of the splats written by the last projection.
 __global__ void k_zero_grads(float4* g, const uint32_t* ctr, int64_t cap) {
+  sequence_begin();
   const int64_t n = 3 * min((int64_t)ctr[kCtrSplats], cap);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -1212,11 +1215,11 @@ int blend_blocks_per_sm(K kernel, int threads, int* cache) {
 }
 
 template <bool kCount, int kWarpsT>
-void launch_fwd(s3r_workspace* ws, const BlendArgs& a, cudaStream_t st) {
+cudaError_t launch_fwd(s3r_workspace* ws, const BlendArgs& a, cudaStream_t st) {
   static thread_local int per_sm = 0;
   constexpr int kThreadsT = 32 * kWarpsT;
   const int g = ws->num_sms * blend_blocks_per_sm(k_blend_fwd<kCount, kWarpsT>, kThreadsT, &per_sm);
-  k_blend_fwd<kCount, kWarpsT><<<g, kThreadsT, 0, st>>>(ws->views, a);
+  return launch_in_sequence(ws, k_blend_fwd<kCount, kWarpsT>, g, kThreadsT, 0, st, ws->views, a);
 }
 
 cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cudaStream_t st) {
@@ -1233,15 +1236,12 @@ cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cu
   // four warps per tile where every tile is resident at once with two (see k_blend_fwd)
   const bool few = ws->views.total_tiles <= ws->num_sms * S3R_BLEND_FWD_BLOCKS;
   KernelTimer timer(ws, kKBlendFwd, st);
-  if (ws->counting) {
-    if (few) launch_fwd<true, 4>(ws, a, st);
-    else launch_fwd<true, 2>(ws, a, st);
-  } else {
-    if (few) launch_fwd<false, 4>(ws, a, st);
-    else launch_fwd<false, 2>(ws, a, st);
-  }
+  if (ws->counting)
+    e = few ? launch_fwd<true, 4>(ws, a, st) : launch_fwd<true, 2>(ws, a, st);
+  else
+    e = few ? launch_fwd<false, 4>(ws, a, st) : launch_fwd<false, 2>(ws, a, st);
   ws->sp_grad_clean = 1;
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_render_bwd(s3r_workspace* ws, const float* bg, const float* dL,
@@ -1253,9 +1253,9 @@ cudaError_t launch_render_bwd(s3r_workspace* ws, const float* bg, const float* d
   // when a backward has used them since
   if (!ws->sp_grad_clean) {
     KernelTimer timer(ws, kKZeroGrads, st);
-    k_zero_grads<<<ws->num_sms * 4, 256, 0, st>>>(reinterpret_cast<float4*>(ws->sp_grad), ws->ctr,
-                                                  ws->cap.max_splats);
-    cudaError_t e0 = cudaGetLastError();
+    const cudaError_t e0 =
+        launch_in_sequence(ws, k_zero_grads, (int64_t)ws->num_sms * 4, 256, 0, st,
+                           reinterpret_cast<float4*>(ws->sp_grad), ws->ctr, ws->cap.max_splats);
     if (e0 != cudaSuccess) return e0;
   }
   ws->sp_grad_clean = 0;
@@ -1271,14 +1271,15 @@ cudaError_t launch_render_bwd(s3r_workspace* ws, const float* bg, const float* d
     return e;
   static thread_local int per_sm[2] = {0, 0};
   KernelTimer timer(ws, kKBlendBwd, st);
-  if (ws->counting) {
-    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_bwd<true>, kBandThreads, &per_sm[1]);
-    k_blend_bwd<true><<<g, kBandThreads, 0, st>>>(ws->views, a);
-  } else {
-    const int g = ws->num_sms * blend_blocks_per_sm(k_blend_bwd<false>, kBandThreads, &per_sm[0]);
-    k_blend_bwd<false><<<g, kBandThreads, 0, st>>>(ws->views, a);
-  }
-  return cudaGetLastError();
+  if (ws->counting)
+    return launch_in_sequence(
+        ws, k_blend_bwd<true>,
+        (int64_t)ws->num_sms * blend_blocks_per_sm(k_blend_bwd<true>, kBandThreads, &per_sm[1]),
+        kBandThreads, 0, st, ws->views, a);
+  return launch_in_sequence(
+      ws, k_blend_bwd<false>,
+      (int64_t)ws->num_sms * blend_blocks_per_sm(k_blend_bwd<false>, kBandThreads, &per_sm[0]),
+      kBandThreads, 0, st, ws->views, a);
 }
 
 }  // namespace s3r

@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_compact(const __grid_constant__
                                                       unsigned long long* lookback,
                                                       uint32_t* __restrict__ sel_bits,
                                                       const CallSetup setup) {
+  sequence_begin();
   __shared__ uint32_t s_bits[kChunkTiles][kWarps][2 * kRounds];   // ballots of the chunk
   __shared__ uint32_t s_off[kChunkTiles * kWarps];   // per (tile, warp): count -> offset in chunk
   __shared__ uint32_t s_tmp[kWarps];
@@ -346,9 +347,8 @@ cudaError_t launch_compact(s3r_workspace* ws, const s3r_scene* sc, const s3r_pos
   c.compose_only = cg.compose_only;
   c.out_count = nullptr;
   KernelTimer timer(ws, kKCompact, st);
-  k_compact<<<cg.grid, kThreads, 0, st>>>(ws->views, vis, n, t, cg.per, ws->selected, ws->ctr,
-                                          ws->lookback, ws->kept_bits, c);
-  return cudaGetLastError();
+  return launch_in_sequence(ws, k_compact, cg.grid, kThreads, 0, st, ws->views, vis, n, t, cg.per,
+                            ws->selected, ws->ctr, ws->lookback, ws->kept_bits, c);
 }
 
 }  // namespace s3r

@@ -68,8 +68,9 @@ static_assert(S3R_PROJECT_MASK_BLOCKS >= 1 && S3R_PROJECT_MASK_BLOCKS * kThreads
               "an SM holds at most 2048 threads");
 __global__ void __launch_bounds__(kThreads, S3R_PROJECT_MASK_BLOCKS) k_project_mask(const __grid_constant__ ViewSet vs,
                                                            ProjArgs a) {
+  sequence_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const InstMat* __restrict__ mats = a.mats;
+  const InstMat* mats = a.mats;
   const int nk = a.n_inst + 1;
   uint32_t* s_off = reinterpret_cast<uint32_t*>(smem_raw);   // [n_inst+2]
   __shared__ uint32_t s_frustum;
@@ -209,10 +210,11 @@ constexpr int kScanItems = 16;
 constexpr int kScanTile = kThreads * kScanItems;
 constexpr int kScanChunkTiles = 16;   // tiles a CTA's shared memory holds the offsets of
 
-__global__ void __launch_bounds__(kThreads) k_splat_scan(const uint32_t* __restrict__ keep_mask,
-                                                         uint32_t* __restrict__ splat_start,
+__global__ void __launch_bounds__(kThreads) k_splat_scan(const uint32_t* keep_mask,
+                                                         uint32_t* splat_start,
                                                          uint32_t* ctr,
                                                          unsigned long long* lookback) {
+  sequence_begin();
   __shared__ uint32_t s_ex[kScanChunkTiles][kThreads];   // thread's offset within the chunk
   __shared__ uint32_t s_tmp[kWarps];
   __shared__ uint32_t s_chunk;
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(kThreads) k_splat_scan(const uint32_t* __restr
       const uint4* p = reinterpret_cast<const uint4*>(keep_mask + j0);
 #pragma unroll
       for (int q = 0; q < kScanItems / 4; ++q) {
-        const uint4 v = __ldg(p + q);
+        const uint4 v = p[q];
         m[4 * q] = v.x; m[4 * q + 1] = v.y; m[4 * q + 2] = v.z; m[4 * q + 3] = v.w;
       }
     } else {
@@ -319,10 +321,11 @@ __global__ void __launch_bounds__(kThreads) k_splat_scan(const uint32_t* __restr
 template <int DEG>
 __global__ void __launch_bounds__(kThreads, 3) k_project_splats(const __grid_constant__ ViewSet vs,
                                                              ProjArgs a) {
+  sequence_begin();
   using St = ShStage<DEG>;
   constexpr int K = St::K;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const InstMat* __restrict__ mats = a.mats;
+  const InstMat* mats = a.mats;
   const int nk = a.n_inst + 1;
   float* s_sh = reinterpret_cast<float*>(smem_raw);                        // [warps][kWords]
   uint32_t* s_off = reinterpret_cast<uint32_t*>(s_sh + kWarps * St::kWords);  // [n_inst+2]
@@ -475,23 +478,25 @@ cudaError_t launch_deg(s3r_workspace* ws, const ProjArgs& a, cudaStream_t st) {
     per_splats = occupancy(k_project_splats<DEG>, smem_splats);
   }
   if (!per_scan) per_scan = occupancy(k_splat_scan, 0);
+  cudaError_t e;
   {
     KernelTimer timer(ws, kKProject, st);
-    k_project_mask<<<ws->num_sms * per_mask, kThreads, smem, st>>>(ws->views, a);
+    e = launch_in_sequence(ws, k_project_mask, (int64_t)ws->num_sms * per_mask, kThreads, smem, st,
+                           ws->views, a);
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   {
     KernelTimer timer(ws, kKSplatScan, st);
-    k_splat_scan<<<(unsigned)scan_ctas((int64_t)ws->num_sms * per_scan), kThreads, 0, st>>>(a.keep_mask, a.splat_start, a.ctr,
-                                                              a.lookback);
+    e = launch_in_sequence(ws, k_splat_scan, scan_ctas((int64_t)ws->num_sms * per_scan), kThreads, 0, st,
+                           a.keep_mask, a.splat_start, a.ctr, a.lookback);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   {
     KernelTimer timer(ws, kKProjectSplats, st);
-    k_project_splats<DEG><<<ws->num_sms * per_splats, kThreads, smem_splats, st>>>(ws->views, a);
+    e = launch_in_sequence(ws, k_project_splats<DEG>, (int64_t)ws->num_sms * per_splats, kThreads,
+                           smem_splats, st, ws->views, a);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

@@ -85,6 +85,7 @@ __device__ __forceinline__ void pose_chain_one(const ViewSet& vs, const float* d
 template <int DEG>
 __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_constant__ ViewSet vs,
                                                           BwdArgs a) {
+  sequence_begin();
   using St = ShStage<DEG>;
   constexpr int K = St::K;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
   // the composed matrices are read through L1 (a CTA touches few instances);
   // shared memory holds each warp's SH rows, the per-(view, instance) matrix
   // adjoints and the camera records (per-lane view indices differ)
-  const InstMat* __restrict__ mats = a.mats;
+  const InstMat* mats = a.mats;
   float* s_sh = reinterpret_cast<float*>(smem_raw);                        // [warps][kWords]
   float* s_dM = s_sh + kWarps * St::kWords;                                // [views][nk][12]
   uint32_t* s_off = reinterpret_cast<uint32_t*>(s_dM + vs.n_views * nk * 12);
@@ -533,8 +534,8 @@ cudaError_t launch_deg(s3r_workspace* ws, const BwdArgs& a, cudaStream_t st) {
   }
   const int per_sm = cached_per_sm;
   KernelTimer timer(ws, kKProjectBwd, st);
-  k_project_bwd<DEG><<<ws->num_sms * per_sm, kThreads, smem, st>>>(ws->views, a);
-  return cudaGetLastError();
+  return launch_in_sequence(ws, k_project_bwd<DEG>, (int64_t)ws->num_sms * per_sm, kThreads, smem, st,
+                            ws->views, a);
 }
 
 }  // namespace

@@ -96,6 +96,7 @@ __device__ __forceinline__ void load_tile(const PassArgs& a, int64_t n, int64_t 
 // per round trip) while those loads are in flight, and write the reordered
 // tile out.
 __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(PassArgs a) {
+  sequence_begin();
   __shared__ uint32_t s_keys[kSortTileKeys];
   __shared__ uint32_t s_vals[kSortTileKeys];
   __shared__ uint32_t s_cnt[kWarps][kRadix];   // per-warp digit counts -> exclusive offsets
@@ -373,6 +374,7 @@ struct TilesArgs {
 
 __global__ void __launch_bounds__(kTilesThreads) k_splat_tiles(const __grid_constant__ ViewSet vs,
                                                               TilesArgs a) {
+  sequence_begin();
   const int64_t n = min((int64_t)a.ctr[kCtrSplats], a.cap);
   const uint32_t lane = lane_id();
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n;
@@ -512,6 +514,7 @@ constexpr int kDupScanTile = kDupThreads * kDupScanItems;   // 4096
 constexpr int kDupScanChunkTiles = 16;
 
 __global__ void __launch_bounds__(kDupThreads) k_dup_scan(DupArgs a) {
+  sequence_begin();
   __shared__ uint32_t s_ex[kDupScanChunkTiles][kDupThreads];   // thread's offset within the chunk
   __shared__ uint32_t s_tmp[kDupThreads / 32];
   __shared__ uint32_t s_chunk;
@@ -696,6 +699,7 @@ struct Cursor {
 };
 
 __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
+  sequence_begin();
   __shared__ uint32_t s_excl[kExpChunk + 1];
   __shared__ uint32_t s_key[kExpChunk];
   __shared__ uint32_t s_val[kExpChunk];
@@ -788,26 +792,27 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
 constexpr int kRangeThreads = 256;
 
 // First position whose key is not below v, among n sorted keys.
-__device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t* __restrict__ keys, uint32_t n,
+__device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t* keys, uint32_t n,
                                                     uint32_t v) {
   uint32_t lo = 0, len = n;   // the answer is in [lo, lo + len]
   while (len >= 8) {
     const uint32_t s = len >> 3;
     uint32_t below = 0;       // of the seven probes at the eighths' last keys
 #pragma unroll
-    for (uint32_t i = 1; i < 8; ++i) below += __ldg(keys + lo + i * s - 1) < v ? 1u : 0u;
+    for (uint32_t i = 1; i < 8; ++i) below += keys[lo + i * s - 1] < v ? 1u : 0u;
     lo += below * s;
     len = below == 7 ? len - 7 * s : s - 1;
   }
   uint32_t below = 0;
 #pragma unroll
-  for (uint32_t i = 0; i < 7; ++i) below += (i < len && __ldg(keys + lo + i) < v) ? 1u : 0u;
+  for (uint32_t i = 0; i < 7; ++i) below += (i < len && keys[lo + i] < v) ? 1u : 0u;
   return lo + below;
 }
 
 __global__ void __launch_bounds__(kRangeThreads) k_tile_ranges(
-    const uint32_t* __restrict__ keys, const uint32_t* ctr, int64_t cap, int tiles,
-    uint2* __restrict__ ranges, uint32_t* class_cnt, uint32_t* __restrict__ class_list) {
+    const uint32_t* keys, const uint32_t* ctr, int64_t cap, int tiles, uint2* ranges,
+    uint32_t* class_cnt, uint32_t* class_list) {
+  sequence_begin();
   __shared__ uint32_t s_cnt[kTileClasses], s_base[kTileClasses];
   const uint32_t K = (uint32_t)min((int64_t)ctr[kCtrDups], cap);
   const uint32_t lane = lane_id();
@@ -869,8 +874,8 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     a.lookback = ws->lookback;
     a.stage = kStageDepth0 + p;
     KernelTimer timer(ws, kKDepth0 + p, st);
-    k_onesweep<<<g_sweep, kSortThreads, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_in_sequence(ws, k_onesweep, g_sweep, kSortThreads, 0, st, a);
+    if (e != cudaSuccess) return e;
   }
   ws->depth_final = 0;
   // expand into (tile, splat) pairs in depth order
@@ -911,19 +916,21 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     t.row_spans = ws->row_spans;
     t.rows_cap = ws->rows_cap;
     t.region = reinterpret_cast<float4*>(ws->sp_region);
-    k_splat_tiles<<<ws->num_sms * tiles_per_sm, kTilesThreads, 0, st>>>(ws->views, t);
+    e = launch_in_sequence(ws, k_splat_tiles, (int64_t)ws->num_sms * tiles_per_sm, kTilesThreads, 0, st,
+                           ws->views, t);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   {
     KernelTimer timer(ws, kKDuplicate, st);
-    k_dup_scan<<<(unsigned)scan_ctas((int64_t)ws->num_sms * dup_per_sm), kDupThreads, 0, st>>>(d);
+    e = launch_in_sequence(ws, k_dup_scan, scan_ctas((int64_t)ws->num_sms * dup_per_sm), kDupThreads, 0,
+                           st, d);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   {
     KernelTimer timer(ws, kKExpand, st);
-    k_dup_expand<<<ws->num_sms * exp_per_sm, kDupThreads, 0, st>>>(d);
+    e = launch_in_sequence(ws, k_dup_expand, (int64_t)ws->num_sms * exp_per_sm, kDupThreads, 0, st, d);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   // tile digits on the pairs
   for (int p = 0; p < ws->tile_passes; ++p) {
     PassArgs a;
@@ -939,8 +946,8 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     a.lookback = ws->lookback;
     a.stage = kStageTile0 + p;
     KernelTimer timer(ws, kKTile0 + p, st);
-    k_onesweep<<<g_sweep, kSortThreads, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_in_sequence(ws, k_onesweep, g_sweep, kSortThreads, 0, st, a);
+    if (e != cudaSuccess) return e;
   }
   ws->dup_final = ws->tile_passes & 1;
   // every tile's range and class (the blend queue)
@@ -950,11 +957,11 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     if (grid > (int64_t)ws->num_sms * 8) grid = (int64_t)ws->num_sms * 8;
     if (grid < 1) grid = 1;
     KernelTimer timer(ws, kKTileRanges, st);
-    k_tile_ranges<<<(unsigned)grid, kRangeThreads, 0, st>>>(
-        ws->dup_key[ws->dup_final], ws->ctr, ws->cap.max_duplicates, tiles, ws->ranges,
-        ws->tile_class_cnt, ws->tile_class_list);
+    e = launch_in_sequence(ws, k_tile_ranges, grid, kRangeThreads, 0, st, ws->dup_key[ws->dup_final],
+                           ws->ctr, ws->cap.max_duplicates, tiles, ws->ranges, ws->tile_class_cnt,
+                           ws->tile_class_list);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace s3r

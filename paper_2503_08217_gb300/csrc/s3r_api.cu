@@ -311,6 +311,7 @@ s3r_status s3r_project(s3r_workspace* ws, const s3r_scene* scene, const s3r_pose
   ws->n_inst = scene->n_inst;
   ws->sh_degree = scene->sh_degree;
   ws->n = scene->n;
+  ws->overlap = scene->n <= kOverlapGaussians;
   int bits = 0;
   while (bits < 32 && ((int64_t)1 << bits) < tiles) ++bits;
   ws->tile_passes = (bits + kRadixBits - 1) / kRadixBits;
