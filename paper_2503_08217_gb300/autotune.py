@@ -53,7 +53,7 @@ PARAMS = (
     Param("S3R_BLEND_FWD_BATCH", "k_blend.cu", (32, 64, 128), "Gaussians staged per batch, blend forward"),
     Param("S3R_BLEND_FWD_BLOCKS", "k_blend.cu", (16, 18, 20, 24), "resident blocks per SM, blend forward"),
     Param("S3R_BLEND_BWD_BATCH", "k_blend.cu", (32, 64, 128), "Gaussians staged per batch, blend backward"),
-    Param("S3R_BLEND_BWD_BLOCKS", "k_blend.cu", (12, 16, 20), "resident blocks per SM, blend backward"),
+    Param("S3R_BLEND_BWD_BLOCKS", "k_blend.cu", (12, 14, 16, 20), "resident blocks per SM, blend backward"),
     Param("S3R_SORT_ITEMS", "s3r_internal.cuh", (11, 15, 18), "keys per thread of a radix tile"),
     Param("S3R_SORT_BLOCKS", "s3r_internal.cuh", (2, 3, 4), "resident onesweep blocks per SM"),
     Param("S3R_SORT_LOOKBACK", "k_sort.cu", (4, 8, 16), "look-back words read per round trip, onesweep"),
