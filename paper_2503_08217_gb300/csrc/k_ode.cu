@@ -23,12 +23,16 @@
 // groups side by side, two steps per tick: two groups recompute the stages of
 // the tick's two steps, a third walks the adjoint through the two steps
 // recomputed one tick earlier, a fourth adds the parameter adjoints of the two
-// steps walked before those, its rows of the sums in registers. They meet at
+// steps walked before those, its rows of the sums in registers, and a ninth warp
+// takes the pose adjoints (sines and cosines) that enter the walk. They meet at
 // one CTA barrier per tick and pass the activations through a ring of three
 // ticks in shared memory.
 //
-// At 120 instances, 400 times, 2 substeps and embedding width 8 the forward and
-// the backward together went from 15.1 to 2.27 ms.
+// At 120 instances, 400 times, 2 substeps and embedding width 8 the forward
+// takes 0.89 ms (570 cycles per evaluation) and the backward 0.98 ms, together
+// 1.88 ms against 15.1 ms. The backward is bound by the adjoint's walk (545
+// cycles per stage): without the ninth warp, its sines and cosines in the
+// recomputing groups, it took 1.37 ms.
 #include "s3r_internal.cuh"
 
 namespace s3r {
@@ -137,13 +141,17 @@ __device__ __forceinline__ void load_eval_weights(EvalWeights& e, const float* _
 // go to h1 and h2 (64 floats of shared memory each). h1 may be rewritten by the
 // next evaluation and h2 after the next evaluation's first barrier, which is
 // where this function writes them, so evaluations follow each other freely.
-__device__ __forceinline__ void eval_f(const EvalWeights& e, const float (&z)[6], float t, int u,
-                                       int bar, float* h1, float* h2, float (&out)[6]) {
+__device__ __forceinline__ void hidden(const EvalWeights& e, const float (&z)[6], float t, int u,
+                                       int bar, float* h1, float* h2) {
   const float a = fmaf(e.w1[2], z[2], fmaf(e.w1[1], z[1], fmaf(e.w1[0], z[0], fmaf(e.wt, t, e.base))));
   const float b = fmaf(e.w1[5], z[5], fmaf(e.w1[4], z[4], e.w1[3] * z[3]));
   h1[u] = tanhf(a + b);
   group_sync(bar);
   h2[u] = tanhf(dot64(h1, e.w2) + e.b2);
+}
+__device__ __forceinline__ void eval_f(const EvalWeights& e, const float (&z)[6], float t, int u,
+                                       int bar, float* h1, float* h2, float (&out)[6]) {
+  hidden(e, z, t, u, bar, h1, h2);
   group_sync(bar);
   six_sums(h2, e.w3, e.b3, (uint32_t)u & 31u, out);
 }
@@ -265,7 +273,7 @@ struct __align__(16) StepSlot {
 };
 static_assert(sizeof(StepSlot) % 16 == 0, "the slots' vectors are read as float4");
 constexpr int kRing = 3, kTickSteps = 2;
-constexpr int kBwdThreads = 4 * kGroup;
+constexpr int kBwdThreads = 4 * kGroup + 32;
 
 // The pose adjoints of state index i (an output time iff i is a multiple of the
 // substeps), for the state's six components.
@@ -285,19 +293,30 @@ __device__ __forceinline__ void pose_adjoint(const OdeArgs& a, int i, int k, flo
   }
 }
 
-// Recomputes the stages of step i (from state i - 1 to state i) into its slot.
-__device__ __forceinline__ void recompute_step(const OdeArgs& a, const EvalWeights& w, int i, int k,
-                                               int u, int bar, StepSlot& s) {
-  const int jj = (i - 1) / a.substeps, sub = (i - 1) - jj * a.substeps;
+// What the recomputation of step i (from state i - 1 to state i) starts from,
+// loaded one tick ahead.
+struct StepStart {
+  float z[6], t0, t1;
+  int sub;
+};
+__device__ __forceinline__ void load_start(const OdeArgs& a, int i, int k, StepStart& s) {
+  const int jj = (i - 1) / a.substeps;
+  s.sub = (i - 1) - jj * a.substeps;
   const float* zs = a.states + 6 * ((size_t)(i - 1) * a.n_inst + k);
-  float z[6], v[6], kk[6];
 #pragma unroll
-  for (int q = 0; q < 6; ++q) z[q] = zs[q];
-  const float t0 = a.times[jj];
-  const float h = (a.times[jj + 1] - t0) / (float)a.substeps;
-  const float t = t0 + (float)sub * h;
+  for (int q = 0; q < 6; ++q) s.z[q] = zs[q];
+  s.t0 = a.times[jj];
+  s.t1 = a.times[jj + 1];
+}
+
+// Recomputes a step's stages into its slot.
+__device__ __forceinline__ void recompute_step(const EvalWeights& w, int substeps, const StepStart& b, int u,
+                                               int bar, StepSlot& s) {
+  const float h = (b.t1 - b.t0) / (float)substeps;
+  const float t = b.t0 + (float)b.sub * h;
+  float v[6], kk[6];
 #pragma unroll
-  for (int q = 0; q < 6; ++q) v[q] = z[q];
+  for (int q = 0; q < 6; ++q) v[q] = b.z[q];
 #pragma unroll
   for (int st = 0; st < 4; ++st) {
     const float ts = st == 0 ? t : (st == 3 ? t + h : t + 0.5f * h);
@@ -307,18 +326,16 @@ __device__ __forceinline__ void recompute_step(const OdeArgs& a, const EvalWeigh
       for (int q = 0; q < 6; ++q) mine = u == q ? v[q] : mine;
       s.x[st][u] = mine;
     }
+    if (st == 3) {   // the last stage's output feeds nothing
+      hidden(w, v, ts, u, bar, s.h1[st], s.h2[st]);
+      break;
+    }
     eval_f(w, v, ts, u, bar, s.h1[st], s.h2[st], kk);
     const float step = st == 2 ? h : 0.5f * h;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) v[q] = fmaf(step, kk[q], z[q]);
+    for (int q = 0; q < 6; ++q) v[q] = fmaf(step, kk[q], b.z[q]);
   }
-  if (u == 0) {
-    float g[6];
-    pose_adjoint(a, i, k, g);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) s.inj[q] = g[q];
-    s.h = h;
-  }
+  if (u == 0) s.h = h;
 }
 
 // Walks the adjoint `ab` of state i back through step i: per stage the reverse
@@ -410,15 +427,31 @@ __global__ void __launch_bounds__(kBwdThreads) k_ode_bwd(OdeArgs a) {
   const int ticks = (n_steps + kTickSteps - 1) / kTickSteps + 2;
   const float* c = a.embed + (size_t)k * a.D;
   const float* p = a.params;
-  // tick n: groups 0 and 1 recompute the steps of tick n, group 2 walks those
-  // of tick n - 1 and group 3 sums those of tick n - 2. Every group runs the
-  // same number of ticks, one CTA barrier each; step s counts from the end.
+  // tick n: groups 0 and 1 recompute the steps of tick n, the ninth warp takes
+  // their pose adjoints, group 2 walks the steps of tick n - 1 and group 3 sums
+  // those of tick n - 2. Every group runs the same number of ticks, one CTA
+  // barrier each; step s counts from the end.
   if (role < kTickSteps) {
     EvalWeights w;
     load_eval_weights(w, p, L, c, u);
+    StepStart now, next;
+    if (role < n_steps) load_start(a, n_steps - role, k, next);
     for (int n = 0; n < ticks; ++n) {
       const int s = n * kTickSteps + role;
-      if (s < n_steps) recompute_step(a, w, n_steps - s, k, u, 1 + role, s_ring[n % kRing][role]);
+      now = next;
+      if (s + kTickSteps < n_steps) load_start(a, n_steps - s - kTickSteps, k, next);
+      if (s < n_steps) recompute_step(w, a.substeps, now, u, 1 + role, s_ring[n % kRing][role]);
+      __syncthreads();
+    }
+  } else if (role == 4) {
+    for (int n = 0; n < ticks; ++n) {
+      const int s = n * kTickSteps + u;
+      if (u < kTickSteps && s < n_steps) {
+        float g[6];
+        pose_adjoint(a, n_steps - s, k, g);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) s_ring[n % kRing][u].inj[q] = g[q];
+      }
       __syncthreads();
     }
   } else if (role == 2) {
