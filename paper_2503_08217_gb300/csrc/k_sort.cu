@@ -235,11 +235,11 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
 //                splat its first output, and every expansion chunk its first
 //                splat.
 //  k_dup_expand: persistent CTAs take fixed chunks of 256 * kExpItems outputs
-//                (2048 at 8); each thread expands kExpItems consecutive
-//                outputs (binary search of the chunk's splat offsets in
-//                shared memory, a walk over the splat's rows to the first
-//                one, then an incremental cursor over rows and splats); the
-//                pairs are staged in shared memory and written coalesced.
+//                (2048 at 8). A lane per splat files each of its rows that falls
+//                into the chunk as a marker at the row's first position in
+//                shared memory (a row's tile ids are consecutive); then every
+//                32 outputs are one coalesced store, each finding its marker
+//                with bit operations on the marked positions.
 constexpr int kDupThreads = 256;
 #ifndef S3R_DUP_EXPAND_ITEMS
 #define S3R_DUP_EXPAND_ITEMS 8   // build-time define the autotuner varies
@@ -248,7 +248,7 @@ constexpr int kExpItems = S3R_DUP_EXPAND_ITEMS;       // outputs per thread per 
 constexpr int kExpChunk = kDupThreads * kExpItems;    // outputs per chunk
 static_assert(kExpChunk >= kDupChunkMin, "the chunk map is sized for chunks of kDupChunkMin");
 static_assert(kExpChunk % 32 == 0, "a chunk clears whole words of contributor bits");
-static_assert(kExpItems <= 14, "above 14 outputs per thread the staged chunk exceeds 48 KB of shared memory");
+static_assert(kExpItems <= 20, "above 20 outputs per thread the staged chunk exceeds 48 KB of shared memory");
 
 constexpr float kSpanPad = 0.05f;        // pixels, on the strips and the column bounds
 
@@ -338,7 +338,8 @@ struct DupArgs {
   const uint2* sp_rect;
   const uint8_t* sp_view;
   const uint32_t* sp_cnt;      // [S] tiles each splat reaches, by depth position
-  const uint32_t* row_spans;   // per row of a rectangle: first | end << 16 (columns)
+  const uint2* row_spans;      // per row of a rectangle: first | end << 16 (columns), and the
+                               // splat's tiles before the row
   const float4* sp_region;     // [S][2] region, by splat id, where sp_rowoff is kNoRows
   uint32_t* dup_key;
   uint32_t* dup_val;
@@ -367,7 +368,7 @@ struct TilesArgs {
   int64_t cap;
   uint32_t* cnt;            // [S] tiles reached, by depth position
   uint4* meta;              // [S][2] expansion records, by depth position
-  uint32_t* row_spans;
+  uint2* row_spans;         // (columns, tiles of the splat before the row)
   int64_t rows_cap;
   float4* region;           // [S][2] by splat id
 };
@@ -375,6 +376,7 @@ struct TilesArgs {
 __global__ void __launch_bounds__(kTilesThreads) k_splat_tiles(const __grid_constant__ ViewSet vs,
                                                               TilesArgs a) {
   sequence_begin();
+  __shared__ uint32_t s_cnt[kTilesThreads];   // tiles of each lane's rows past the inline ones
   const int64_t n = min((int64_t)a.ctr[kCtrSplats], a.cap);
   const uint32_t lane = lane_id();
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n;
@@ -430,34 +432,58 @@ __global__ void __launch_bounds__(kTilesThreads) k_splat_tiles(const __grid_cons
           head[r] = c.x | (c.y << 16);
           cnt += c.y - c.x;
         }
-    // the warp: the further rows of its taller splats, one splat at a time,
-    // one row per lane (a per-lane loop would wait on the tallest splat)
-    uint32_t tall = __ballot_sync(0xffffffffu, need != 0u);
-    while (tall) {
-      const int b = __ffs(tall) - 1;
-      tall &= tall - 1;
-      Region gb;
-      gb.u = __shfl_sync(0xffffffffu, g.u, b);
-      gb.v = __shfl_sync(0xffffffffu, g.v, b);
-      gb.B = __shfl_sync(0xffffffffu, g.B, b);
-      gb.inv_A = __shfl_sync(0xffffffffu, g.inv_A, b);
-      gb.LA = __shfl_sync(0xffffffffu, g.LA, b);
-      gb.det = __shfl_sync(0xffffffffu, g.det, b);
-      gb.ye = __shfl_sync(0xffffffffu, g.ye, b);
-      gb.xe = __shfl_sync(0xffffffffu, g.xe, b);
-      gb.s = __shfl_sync(0xffffffffu, g.s, b);
-      const uint32_t wb = __shfl_sync(0xffffffffu, w, b), hb = __shfl_sync(0xffffffffu, h, b);
-      const uint64_t ob = __shfl_sync(0xffffffffu, (unsigned long long)off, b);
-      const bool tb = __shfl_sync(0xffffffffu, (int)table, b) != 0;
-      uint32_t part = 0;
-      for (uint32_t r = kInlineRows + lane; r < hb; r += 32) {
-        const uint2 c = row_span(gb, r, wb);
-        part += c.y - c.x;
-        if (tb) a.row_spans[ob + (r - kInlineRows)] = c.x | (c.y << 16);
-      }
+    // the warp: the further rows of its taller splats as one list, a row per
+    // lane; row t of the list belongs to the first lane whose running count
+    // exceeds t, and the lists of a warp's splats stand together in the table.
+    // (A splat at a time, a lane per row, kept 14 lanes of 32 idle.)
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (total) {   // warp-uniform
+      s_cnt[threadIdx.x] = 0u;
+      __syncwarp();
+      for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        int o = 0;   // owner: lanes below it have incl <= t
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-      if (lane == (uint32_t)b) cnt += part;
+        for (int step = 16; step > 0; step >>= 1) {
+          const uint32_t x = __shfl_sync(0xffffffffu, incl, min(o + step - 1, 31));
+          if (x <= t) o += step;
+        }
+        o = min(o, 31);
+        Region gb;
+        gb.u = __shfl_sync(0xffffffffu, g.u, o);
+        gb.v = __shfl_sync(0xffffffffu, g.v, o);
+        gb.B = __shfl_sync(0xffffffffu, g.B, o);
+        gb.inv_A = __shfl_sync(0xffffffffu, g.inv_A, o);
+        gb.LA = __shfl_sync(0xffffffffu, g.LA, o);
+        gb.det = __shfl_sync(0xffffffffu, g.det, o);
+        gb.ye = __shfl_sync(0xffffffffu, g.ye, o);
+        gb.xe = __shfl_sync(0xffffffffu, g.xe, o);
+        gb.s = __shfl_sync(0xffffffffu, g.s, o);
+        const uint32_t wb = __shfl_sync(0xffffffffu, w, o);
+        const uint32_t before = __shfl_sync(0xffffffffu, incl - need, o);
+        const bool tb = __shfl_sync(0xffffffffu, (int)table, o) != 0;
+        uint2 c = make_uint2(0u, 0u);
+        if (t < total) c = row_span(gb, kInlineRows + (t - before), wb);
+        // the splat's tiles before this row: its inline rows', its rows' of
+        // earlier rounds, and its rows' of the lanes before in this round
+        const uint32_t len = c.y - c.x;
+        uint32_t run = len;
+#pragma unroll
+        for (int st = 1; st < 32; st <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, run, st);
+          if (lane >= (uint32_t)st) run += y;
+        }
+        const uint32_t first = before > t0 ? before - t0 : 0u;   // its first lane here
+        const uint32_t skip = __shfl_sync(0xffffffffu, run - len, (int)min(first, 31u));
+        const uint32_t inline_cnt = __shfl_sync(0xffffffffu, cnt, o);
+        uint32_t* far_cnt = &s_cnt[(threadIdx.x & ~31u) + o];
+        if (t < total && tb)
+          a.row_spans[wbase + t] = make_uint2(c.x | (c.y << 16), inline_cnt + *far_cnt + (run - len - skip));
+        __syncwarp();
+        if (len) atomicAdd(far_cnt, len);
+        __syncwarp();
+      }
+      cnt += s_cnt[threadIdx.x];
     }
     if (!live) continue;
     const ViewInfo& vi = vs.v[sview & 0x7f];   // bit 7: Eq. 7 moved
@@ -611,167 +637,180 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_scan(DupArgs a) {
   }
 }
 
-// Per-thread run-length counting of the radix digits of a key sequence: one
-// shared atomic per run of equal digits (consecutive outputs walk a tile
-// row, so the higher digits repeat for many outputs).
-struct DigitRuns {
-  uint32_t d[4], n[4];
-  __device__ __forceinline__ void init() {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) { d[p] = 0; n[p] = 0; }
-  }
-  __device__ __forceinline__ void add(uint32_t (*s_hist)[kRadix], uint32_t key, int passes) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      if (p >= passes) break;
-      const uint32_t dg = (key >> (8 * p)) & 0xffu;
-      if (dg != d[p]) {
-        if (n[p]) atomicAdd(&s_hist[p][d[p]], n[p]);
-        d[p] = dg;
-        n[p] = 0;
-      }
-      ++n[p];
-    }
-  }
-  __device__ __forceinline__ void flush(uint32_t (*s_hist)[kRadix], int passes) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-      if (p < passes && n[p]) atomicAdd(&s_hist[p][d[p]], n[p]);
-  }
+// A row of one splat's tiles falling into a chunk: `len` pairs from output `o`
+// on, their tile ids consecutive from `key`. The part inside the chunk is filed
+// as one marker at its first position: the splat, and the tile id less the
+// position, so that the pairs of a marker are its value plus their positions.
+// The digits above the lowest are counted here, a piece of equal digits at a
+// time (pieces end at multiples of 256); the lowest is counted by the pairs.
+struct ExpandChunk {
+  uint32_t O0, O1;
+  uint32_t* key;            // [kExpChunk] tile id less position, at marked positions
+  uint32_t* val;            // [kExpChunk] splat
+  uint32_t* mark;           // [kExpChunk / 32] bits
+  uint32_t (*hist)[kRadix];
+  int passes;
 };
-
-// Position in the expansion of one splat: row r of its rectangle, column c in
-// the row's interval [.., ce). Rows past the rectangle (an inconsistent count,
-// which the shared row function rules out) stay on its last row, so every key
-// is a tile of the splat's view.
-struct Cursor {
-  const uint32_t* row_spans;
-  const float4* region;
-  uint32_t sp, corner, gx, w, h, off;
-  uint32_t head[kInlineRows];
-  uint32_t r, c, ce, row_tile;
-  __device__ __forceinline__ void load(const uint4* m, const DupArgs& a) {
-    row_spans = a.row_spans;
-    region = a.sp_region;
-    const uint4 d = m[0], e = m[1];
-    sp = d.x;
-    corner = d.y;
-    gx = d.z & 0xffffu;
-    w = d.z >> 16;
-    h = d.w;
-    off = e.x;
-    head[0] = e.y;
-    head[1] = e.z;
-    head[2] = e.w;
+__device__ __forceinline__ void file_row(const ExpandChunk& c, uint32_t splat, uint32_t o, uint32_t len,
+                                         uint32_t key) {
+  const uint32_t lo = max(o, c.O0), hi = min(o + len, c.O1);
+  if (lo >= hi) return;
+  const uint32_t pos = lo - c.O0;
+  uint32_t k = key + (lo - o);
+  c.key[pos] = k - pos;
+  c.val[pos] = splat;
+  atomicOr(c.mark + (pos >> 5), 1u << (pos & 31u));
+  if (c.passes < 2) return;
+  for (uint32_t left = hi - lo; left > 0;) {
+    const uint32_t n = min(left, kRadix - (k & (kRadix - 1)));
+    for (int p = 1; p < c.passes; ++p) atomicAdd(&c.hist[p][(k >> (8 * p)) & 0xffu], n);
+    k += n;
+    left -= n;
   }
-  // rows past the inline ones: the row table, or (where it had no room) the
-  // stored region through the same function that counted them
-  __device__ __forceinline__ uint32_t far_row(uint32_t row) const {
-    if (off != kNoRows) return row_spans[off + row - kInlineRows];
-    const Region g = region_load(region[2 * (size_t)sp], region[2 * (size_t)sp + 1]);
-    const uint2 s = row_span(g, row, w);
-    return s.x | (s.y << 16);
-  }
-  __device__ __forceinline__ void set_row(uint32_t rr) {
-    r = rr;
-    const uint32_t row = min(r, h - 1u);
-    static_assert(kInlineRows == 3, "the selects below take rows 0..2 from registers");
-    const uint32_t e = row == 0 ? head[0] : row == 1 ? head[1] : row == 2 ? head[2] : far_row(row);
-    c = e & 0xffffu;
-    ce = e >> 16;
-    row_tile = corner + row * gx;
-  }
-  // the k-th output of the splat (k < its count)
-  __device__ __forceinline__ void seek(uint32_t k) {
-    set_row(0);
-    while (r + 1 < h && k >= ce - c) {
-      k -= ce - c;
-      set_row(r + 1);
-    }
-    c += min(k, ce > c ? ce - c - 1 : 0u);
-  }
-  __device__ __forceinline__ void next() {
-    if (++c < ce) return;
-    do {
-      set_row(r + 1);
-    } while (c >= ce && r + 1 < h);
-  }
-};
+}
 
 __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
   sequence_begin();
-  __shared__ uint32_t s_excl[kExpChunk + 1];
   __shared__ uint32_t s_key[kExpChunk];
   __shared__ uint32_t s_val[kExpChunk];
-  __shared__ uint32_t s_chunk, s_q0, s_q1;
+  __shared__ uint32_t s_mark[kExpChunk / 32];
+  __shared__ uint32_t s_chunk;
   __shared__ uint32_t s_hist[4][kRadix];
+  constexpr int kWordsPerWarp = kExpChunk / 32 / (kDupThreads / 32);
   for (int i = threadIdx.x; i < 4 * kRadix; i += kDupThreads) (&s_hist[0][0])[i] = 0;
-  const int64_t n = min((int64_t)a.ctr[kCtrSplats], a.cap_splats);
   const int64_t total = min((int64_t)a.ctr[kCtrDups], a.cap_dups);
   const int64_t n_chunks = (total + kExpChunk - 1) / kExpChunk;
+  const uint32_t lane = lane_id();
+  const int warp = threadIdx.x >> 5;
   for (;;) {
     if (threadIdx.x == 0) s_chunk = atomicAdd(a.ctr + kCtrTileBase + kStageExpand, 1u);
+    for (int i = threadIdx.x; i < kExpChunk / 32; i += kDupThreads) s_mark[i] = 0u;
     __syncthreads();
     const int64_t chunk = s_chunk;
     if (chunk >= n_chunks) break;
-    const uint32_t O0 = (uint32_t)(chunk * kExpChunk);
-    const uint32_t O1 = (uint32_t)min((int64_t)O0 + kExpChunk, total);   // exclusive
-    // the chunk's splats: from the one holding its first output to (at most)
-    // the one holding the next chunk's first output, from the scan's map
-    if (threadIdx.x == 0) {
-      s_q0 = a.dup_chunk[chunk];
-      s_q1 = a.dup_chunk[chunk + 1];
-    }
-    __syncthreads();
-    // at most one splat per output has outputs here, and splats without any
-    // sort after all of them, so kExpChunk bounds the count
-    const int q0 = (int)s_q0, nq = min((int)s_q1 - q0 + 1, kExpChunk);
-    for (int i = threadIdx.x; i <= nq; i += kDupThreads) s_excl[i] = a.dup_excl[q0 + i];
-    __syncthreads();
-    // kExpItems consecutive outputs per thread
-    const uint32_t o0 = O0 + threadIdx.x * kExpItems;
-    if (o0 < O1) {
-      int lo = 0, hi = nq;            // last local q with s_excl[q] <= o0
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (s_excl[mid] <= o0) lo = mid; else hi = mid;
+    ExpandChunk c;
+    c.O0 = (uint32_t)(chunk * kExpChunk);
+    c.O1 = (uint32_t)min((int64_t)c.O0 + kExpChunk, total);   // exclusive
+    c.key = s_key;
+    c.val = s_val;
+    c.mark = s_mark;
+    c.hist = s_hist;
+    c.passes = a.tile_passes;
+    // 1. the chunk's splats, from the one holding its first output to (at most)
+    //    the one holding the next chunk's first output (the scan's map), a lane
+    //    each: the inline rows by their lane, the further rows of the taller
+    //    ones by the warp, a row per lane
+    const uint32_t q0 = a.dup_chunk[chunk], q1 = a.dup_chunk[chunk + 1];
+    for (uint32_t qb = q0 + warp * 32; qb <= q1; qb += kDupThreads) {
+      const uint32_t q = qb + lane;
+      uint32_t o = 0, o0 = 0, corner = 0, gx = 0, w = 0, h = 0, off = 0, sp = 0;
+      if (q <= q1) {
+        const uint4 d = a.dup_meta[2 * (size_t)q], e = a.dup_meta[2 * (size_t)q + 1];
+        o0 = o = a.dup_excl[q];
+        sp = d.x;
+        corner = d.y;
+        gx = d.z & 0xffffu;
+        w = d.z >> 16;
+        h = d.w;
+        off = e.x;
+        const uint32_t head[kInlineRows] = {e.y, e.z, e.w};
+#pragma unroll
+        for (uint32_t r = 0; r < (uint32_t)kInlineRows; ++r)
+          if (r < h) {
+            const uint32_t first = head[r] & 0xffffu, len = (head[r] >> 16) - first;
+            file_row(c, sp, o, len, corner + r * gx + first);
+            o += len;
+          }
       }
-      int q = lo;
-      const uint32_t oe = min(o0 + kExpItems, O1);
-      // cursor: splat q, its row r with columns [c, ce), tile id of column 0 of row r
-      Cursor cur;
-      cur.load(a.dup_meta + 2 * (q0 + q), a);
-      cur.seek(o0 - s_excl[q]);
-      uint32_t q_end = s_excl[q + 1];
-      DigitRuns runs;
-      runs.init();
-      for (uint32_t o = o0; o < oe; ++o) {
-        while (o >= q_end) {
-          ++q;
-          q_end = s_excl[q + 1];
-          cur.load(a.dup_meta + 2 * (q0 + q), a);
-          cur.seek(0);
+      // the further rows in the table, as one list (see k_splat_tiles)
+      const bool tall = h > (uint32_t)kInlineRows && o < c.O1;
+      const uint32_t need = tall && off != kNoRows ? h - kInlineRows : 0u;
+      uint32_t incl = need;
+#pragma unroll
+      for (int st = 1; st < 32; st <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, st);
+        if (lane >= (uint32_t)st) incl += y;
+      }
+      const uint32_t rows = __shfl_sync(0xffffffffu, incl, 31);
+      for (uint32_t t0 = 0; t0 < rows; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        int b = 0;   // owner: lanes below it have incl <= t
+#pragma unroll
+        for (int st = 16; st > 0; st >>= 1) {
+          const uint32_t x = __shfl_sync(0xffffffffu, incl, min(b + st - 1, 31));
+          if (x <= t) b += st;
         }
-        const uint32_t key = cur.row_tile + cur.c;
-        s_key[o - O0] = key;
-        s_val[o - O0] = cur.sp;
-        runs.add(s_hist, key, a.tile_passes);
-        cur.next();
+        b = min(b, 31);
+        const uint32_t r = t - __shfl_sync(0xffffffffu, incl - need, b);   // past the inline ones
+        const uint32_t fb = __shfl_sync(0xffffffffu, off, b), gb = __shfl_sync(0xffffffffu, gx, b);
+        const uint32_t cb = __shfl_sync(0xffffffffu, corner, b), sb = __shfl_sync(0xffffffffu, sp, b);
+        const uint32_t ob = __shfl_sync(0xffffffffu, o0, b);
+        if (t < rows) {
+          const uint2 row = a.row_spans[fb + r];
+          const uint32_t first = row.x & 0xffffu;
+          file_row(c, sb, ob + row.y, (row.x >> 16) - first, cb + (r + kInlineRows) * gb + first);
+        }
       }
-      runs.flush(s_hist, a.tile_passes);
+      // and those the table had no room for: from the stored region, through the
+      // function that counted them, a splat at a time
+      uint32_t loose = __ballot_sync(0xffffffffu, tall && off == kNoRows);
+      while (loose) {
+        const int b = __ffs(loose) - 1;
+        loose &= loose - 1;
+        const uint32_t hb = __shfl_sync(0xffffffffu, h, b), gb = __shfl_sync(0xffffffffu, gx, b);
+        const uint32_t cb = __shfl_sync(0xffffffffu, corner, b), sb = __shfl_sync(0xffffffffu, sp, b);
+        const uint32_t wb = __shfl_sync(0xffffffffu, w, b);
+        uint32_t ob = __shfl_sync(0xffffffffu, o, b);
+        const Region g = region_load(a.sp_region[2 * (size_t)sb], a.sp_region[2 * (size_t)sb + 1]);
+        for (uint32_t r0 = kInlineRows; r0 < hb && ob < c.O1; r0 += 32) {
+          const uint32_t r = r0 + lane;
+          const uint2 row = r < hb ? row_span(g, r, wb) : make_uint2(0u, 0u);
+          const uint32_t len = row.y - row.x;
+          uint32_t run = len;
+#pragma unroll
+          for (int st = 1; st < 32; st <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, run, st);
+            if (lane >= (uint32_t)st) run += y;
+          }
+          file_row(c, sb, ob + run - len, len, cb + r * gb + row.x);
+          ob += __shfl_sync(0xffffffffu, run, 31);
+        }
+      }
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < O1 - O0; i += kDupThreads) {
-      __stcs(a.dup_key + O0 + i, s_key[i]);
-      __stcs(a.dup_val + O0 + i, s_val[i]);
+    // 2. the pairs, 32 positions at a time: a pair belongs to the last marker at
+    //    or before its position (the chunk's first position has one)
+    const uint32_t n_here = c.O1 - c.O0;
+    uint32_t word = (uint32_t)(warp * kWordsPerWarp);
+    uint32_t carry = 0;   // last marked position before the word
+    for (uint32_t x = word; x > 0;) {
+      const uint32_t bits = s_mark[--x];
+      if (bits) {
+        carry = x * 32u + 31u - __clz(bits);
+        break;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kWordsPerWarp; ++i, ++word) {
+      const uint32_t bits = s_mark[word], pos = word * 32u + lane;
+      const uint32_t at_or_before = bits & (0xffffffffu >> (31u - lane));
+      const uint32_t m = at_or_before ? word * 32u + 31u - __clz(at_or_before) : carry;
+      if (pos < n_here) {
+        const uint32_t key = s_key[m] + pos;
+        __stcs(a.dup_key + c.O0 + pos, key);
+        __stcs(a.dup_val + c.O0 + pos, s_val[m]);
+        atomicAdd(&s_hist[0][key & 0xffu], 1u);
+      }
+      if (bits) carry = word * 32u + 31u - __clz(bits);
     }
     // the contributor bits of the chunk's pair positions, for the forward: as
     // many words as there are pairs, where clearing them for the whole pair
     // capacity in the tile-range launch (a few CTAs on small images) took most
     // of that launch
     for (int b = 0; b < a.bands; ++b)
-      for (uint32_t i = threadIdx.x; i < (O1 - O0 + 31u) / 32u; i += kDupThreads)
-        a.contrib[b * a.contrib_words + O0 / 32u + i] = 0u;
+      for (uint32_t i = threadIdx.x; i < (n_here + 31u) / 32u; i += kDupThreads)
+        a.contrib[b * a.contrib_words + c.O0 / 32u + i] = 0u;
+    __syncthreads();   // the markers are rewritten by the next chunk
   }
   __syncthreads();
   for (int i = threadIdx.x; i < a.tile_passes * kRadix; i += kDupThreads) {

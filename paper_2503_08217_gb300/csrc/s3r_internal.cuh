@@ -181,7 +181,7 @@ struct s3r_workspace {
   uint32_t* dup_meta;       // [S] x 8: expansion record of each splat, depth order
   uint32_t* sp_tiles;       // [S] tiles of its rectangle a splat's alpha region reaches, depth order
   float* sp_region;         // [S] x 8: that region, where the row table had no room
-  uint32_t* row_spans;      // [rows_cap] column interval of one rectangle row
+  uint2* row_spans;         // [rows_cap] column interval of one rectangle row, and the splat's tiles before it
   int64_t rows_cap;
   uint32_t* dup_chunk;      // [K/kDupChunkMin + 2] sorted splat holding the first pair of each expansion chunk
   uint32_t* contrib;        // [4][K/32 + 2] bit per (warp block, sorted pair): blended in the forward
