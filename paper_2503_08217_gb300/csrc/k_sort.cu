@@ -235,20 +235,21 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
 //                splat its first output, and every expansion chunk its first
 //                splat.
 //  k_dup_expand: persistent CTAs take fixed chunks of 256 * kExpItems outputs
-//                (2048 at 8). A lane per splat files each of its rows that falls
+//                (3072 at 12: 0.137 ms at the surround rig, 2048 0.150, 1024 0.191,
+//                4096 0.148). A lane per splat files each of its rows that falls
 //                into the chunk as a marker at the row's first position in
 //                shared memory (a row's tile ids are consecutive); then every
 //                32 outputs are one coalesced store, each finding its marker
 //                with bit operations on the marked positions.
 constexpr int kDupThreads = 256;
 #ifndef S3R_DUP_EXPAND_ITEMS
-#define S3R_DUP_EXPAND_ITEMS 8   // build-time define the autotuner varies
+#define S3R_DUP_EXPAND_ITEMS 12   // build-time define the autotuner varies
 #endif
 constexpr int kExpItems = S3R_DUP_EXPAND_ITEMS;       // outputs per thread per chunk
 constexpr int kExpChunk = kDupThreads * kExpItems;    // outputs per chunk
 static_assert(kExpChunk >= kDupChunkMin, "the chunk map is sized for chunks of kDupChunkMin");
 static_assert(kExpChunk % 32 == 0, "a chunk clears whole words of contributor bits");
-static_assert(kExpItems <= 20, "above 20 outputs per thread the staged chunk exceeds 48 KB of shared memory");
+static_assert(kExpItems <= 14, "above 14 outputs per thread the larger chunks measured slower");
 
 constexpr float kSpanPad = 0.05f;        // pixels, on the strips and the column bounds
 
@@ -373,23 +374,37 @@ struct TilesArgs {
   float4* region;           // [S][2] by splat id
 };
 
-__global__ void __launch_bounds__(kTilesThreads) k_splat_tiles(const __grid_constant__ ViewSet vs,
+// Four blocks per SM (61 registers): 0.103 ms at the surround rig (4.16M splats),
+// three 0.114, five 0.108; without the loads ahead 0.115.
+__global__ void __launch_bounds__(kTilesThreads, 4) k_splat_tiles(const __grid_constant__ ViewSet vs,
                                                               TilesArgs a) {
   sequence_begin();
   __shared__ uint32_t s_cnt[kTilesThreads];   // tiles of each lane's rows past the inline ones
   const int64_t n = min((int64_t)a.ctr[kCtrSplats], a.cap);
   const uint32_t lane = lane_id();
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n;
-       base += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t i_first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  uint32_t sp_next = i_first < n ? a.sorted[i_first] : 0u;
+  uint32_t sp_after = i_first + stride < n ? a.sorted[i_first + stride] : 0u;
+  uint4 t0_next = make_uint4(0u, 0u, 0u, 0u), t1_next = t0_next;
+  if (i_first < n) {
+    t0_next = a.tin[2 * (size_t)sp_next];
+    t1_next = a.tin[2 * (size_t)sp_next + 1];
+  }
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n; base += stride) {
     const int64_t i = base + threadIdx.x;   // depth position
     const bool live = i < n;
-    const uint32_t sp = live ? a.sorted[i] : 0u;
-    // the packed inputs: one 32-byte sector per splat
-    uint4 t0 = make_uint4(0u, 0u, 0u, 0u), t1 = make_uint4(0u, 0u, 0u, 0u);
-    if (live) {
-      t0 = a.tin[2 * (size_t)sp];
-      t1 = a.tin[2 * (size_t)sp + 1];
+    // the packed inputs: one 32-byte sector per splat, gathered by the sorted id;
+    // the next round's are on their way while this one's rows are computed, the
+    // ids a round further ahead
+    const uint32_t sp = sp_next;
+    const uint4 t0 = t0_next, t1 = t1_next;
+    sp_next = sp_after;
+    if (i + stride < n) {
+      t0_next = a.tin[2 * (size_t)sp_next];
+      t1_next = a.tin[2 * (size_t)sp_next + 1];
     }
+    sp_after = i + 2 * stride < n ? a.sorted[i + 2 * stride] : 0u;
     const float2 sxy = make_float2(__uint_as_float(t0.x), __uint_as_float(t0.y));
     const float4 sco = make_float4(__uint_as_float(t0.z), __uint_as_float(t0.w),
                                    __uint_as_float(t1.x), __uint_as_float(t1.y));
