@@ -12,9 +12,9 @@
 // atomics: a Gaussian has one thread). The SH rows are
 // read, and their adjoints added, through shared memory with coalesced
 // accesses of the whole warp.
-// Adjoints of the composed 3x4 matrices are summed per (view, instance) in
-// shared memory and flushed once per CTA; the last CTA to finish then maps
-// them to the pose: dP = V_rot^T dW, and through R(q) to (dq, dt).
+// Adjoints of the composed 3x4 matrices are added to the sums of their (view,
+// instance) in global memory, three vector reductions a Gaussian and pass; the
+// last CTA to finish then maps them to the pose: dP = V_rot^T dW, and through R(q) to (dq, dt).
 #include "s3r_math.cuh"
 
 namespace s3r {
@@ -82,6 +82,22 @@ __device__ __forceinline__ void pose_chain_one(const ViewSet& vs, const float* d
   }
 }
 
+// Adds a matrix adjoint (dA | db, rows of four, 16-byte aligned) to the sums at
+// dst. The reductions are done in L2, without an answer. (Sums in shared memory,
+// one float at a time: such an add retries until no other lane's came between,
+// and a warp's lanes mostly share an instance, so a batch of one instance's
+// Gaussians took about 25 us: 1001 x 563, 5 instances near the camera, 63 ->
+// 39 us a view with the grouped SH sums below; one 1080p view 94 -> 76 us; the
+// surround rig 415 -> 387 us. Sums over the warp's lanes first took 22 us on the
+// small view, but 438 us at the rig: registers spilled.)
+__device__ __forceinline__ void add_matrix_adjoint(float* dst, const float (&dA)[9], const float (&db)[3]) {
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 4 * r), "f"(dA[3 * r]),
+                 "f"(dA[3 * r + 1]), "f"(dA[3 * r + 2]), "f"(db[r])
+                 : "memory");
+}
+
 template <int DEG>
 __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_constant__ ViewSet vs,
                                                           BwdArgs a) {
@@ -91,12 +107,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nk = a.n_inst + 1;
   // the composed matrices are read through L1 (a CTA touches few instances);
-  // shared memory holds each warp's SH rows, the per-(view, instance) matrix
-  // adjoints and the camera records (per-lane view indices differ)
+  // shared memory holds each warp's SH rows and the camera records (per-lane
+  // view indices differ)
   const InstMat* mats = a.mats;
   float* s_sh = reinterpret_cast<float*>(smem_raw);                        // [warps][kWords]
-  float* s_dM = s_sh + kWarps * St::kWords;                                // [views][nk][12]
-  uint32_t* s_off = reinterpret_cast<uint32_t*>(s_dM + vs.n_views * nk * 12);
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(s_sh + kWarps * St::kWords);
   __shared__ ViewInfo s_views[S3R_MAX_VIEWS];
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(vs.v);
@@ -104,7 +119,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
     const int words = vs.n_views * (int)(sizeof(ViewInfo) / 4);
     for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = src[i];
   }
-  for (int i = threadIdx.x; i < vs.n_views * nk * 12; i += blockDim.x) s_dM[i] = 0.f;
   for (int i = threadIdx.x; i < nk + 1; i += blockDim.x) s_off[i] = (uint32_t)a.inst_off[i];
   __syncthreads();
   const int warp = threadIdx.x >> 5;
@@ -298,16 +312,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
         dA[3 * r] += dp[r] * mv[0]; dA[3 * r + 1] += dp[r] * mv[1]; dA[3 * r + 2] += dp[r] * mv[2];
         db[r] += dp[r];
       }
-      if (k > 0) {
-        float* dst = s_dM + (v * nk + k) * 12;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          atomicAdd(dst + 4 * r, dA[3 * r]);
-          atomicAdd(dst + 4 * r + 1, dA[3 * r + 1]);
-          atomicAdd(dst + 4 * r + 2, dA[3 * r + 2]);
-          atomicAdd(dst + 4 * r + 3, db[r]);
-        }
-      }
+      if (k > 0) add_matrix_adjoint(a.pose_dM + (v * nk + k) * 12, dA, db);
     }
 
     // ---- RS = R diag(s), s = exp(log s), R = R(q/|q|)
@@ -409,16 +414,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
         }
       }
 
-      if (DEG > 0 && k > 0) {
-        float* dst = s_dM + (v * nk + k) * 12;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          atomicAdd(dst + 4 * r, dA[3 * r]);
-          atomicAdd(dst + 4 * r + 1, dA[3 * r + 1]);
-          atomicAdd(dst + 4 * r + 2, dA[3 * r + 2]);
-          atomicAdd(dst + 4 * r + 3, db[r]);
-        }
-      }
+      if (DEG > 0 && k > 0) add_matrix_adjoint(a.pose_dM + (v * nk + k) * 12, dA, db);
     }
     if (a.g.means) {
       float* p = a.g.means + 3 * (size_t)gid;
@@ -459,24 +455,34 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
           }
         }
       } else {
+        // nine elements a group; accumulating, a group's old values are loaded
+        // before its first store: one round trip per group, not per element
+        constexpr int kTogether = 9;
+#pragma unroll 1
+        for (int it0 = 0; it0 < St::kRow; it0 += kTogether) {
+          float old[kTogether];
+          float* at[kTogether];
 #pragma unroll
-        for (int it = 0; it < St::kRow; ++it) {
-          const int idx = it * 32 + (int)lane;
-          const int g = idx / St::kRow, qd = idx - g * St::kRow;
-          const uint32_t gg = __shfl_sync(0xffffffffu, gid, g);
-          if ((live >> g) & 1u) {
-            float* q = a.g.sh + (size_t)gg * St::kRow + qd;
-            *q = a.overwrite ? my_sh[g * St::kPitch + qd] : *q + my_sh[g * St::kPitch + qd];
+          for (int e = 0; e < kTogether; ++e) {
+            const int idx = (it0 + e) * 32 + (int)lane;
+            const int g = min(idx / St::kRow, 31), qd = idx - g * St::kRow;
+            const uint32_t gg = __shfl_sync(0xffffffffu, gid, g);
+            const bool on = it0 + e < St::kRow && ((live >> g) & 1u);
+            at[e] = on ? a.g.sh + (size_t)gg * St::kRow + qd : nullptr;
+            old[e] = on && !a.overwrite ? *at[e] : 0.f;
           }
+#pragma unroll
+          for (int e = 0; e < kTogether; ++e)
+            if (at[e]) {
+              const int idx = (it0 + e) * 32 + (int)lane;
+              const int g = idx / St::kRow, qd = idx - g * St::kRow;
+              const float d = my_sh[g * St::kPitch + qd];
+              *at[e] = a.overwrite ? d : old[e] + d;
+            }
         }
       }
     }
     __syncwarp();
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < vs.n_views * nk * 12; i += blockDim.x) {
-    const int k = (i / 12) % nk;
-    if (k > 0 && s_dM[i] != 0.f) atomicAdd(a.pose_dM + i, s_dM[i]);
   }
   // the last CTA to finish maps the summed matrix adjoints to the poses, then
   // clears the sums for the next call (they start at zero with the workspace)
@@ -503,7 +509,7 @@ template <int DEG>
 cudaError_t launch_deg(s3r_workspace* ws, const BwdArgs& a, cudaStream_t st) {
   const int nk = ws->n_inst + 1;
   const size_t smem = sizeof(float) * kWarps * ShStage<DEG>::kWords +
-                      (size_t)ws->n_views * nk * 12 * sizeof(float) + sizeof(uint32_t) * (nk + 1) + 16;
+                      sizeof(uint32_t) * (nk + 1) + 16;
   // The dynamic shared-memory limit is a property of the function, shared by all
   // threads, and the size depends on the scene: it is raised once to the most
   // the device allows, so that no thread's scene lowers it under another's.
