@@ -13,8 +13,9 @@
 // read, and their adjoints added, through shared memory with coalesced
 // accesses of the whole warp.
 // Adjoints of the composed 3x4 matrices are added to the sums of their (view,
-// instance) in global memory, three vector reductions a Gaussian and pass; the
-// last CTA to finish then maps them to the pose: dP = V_rot^T dW, and through R(q) to (dq, dt).
+// instance) in global memory, three vector reductions a Gaussian and pass, in
+// one of several copies of the sums; a second kernel adds the copies up and maps
+// them to the pose: dP = V_rot^T dW, and through R(q) to (dq, dt).
 #include "s3r_math.cuh"
 
 namespace s3r {
@@ -43,38 +44,86 @@ struct BwdArgs {
   LodArgs L;
   int64_t cap_splats;
   uint32_t* ctr;
-  float* pose_dM;          // [n_views][n_inst+1][12]
+  float* pose_dM;          // [pose_copies][n_views][n_inst+1][12]
+  int pose_copies;
   s3r_grads g;
   const InstMat* mats;     // composed by the forward's compaction (same poses)
   int overwrite;           // S3R_GRAD_OVERWRITE: write the rows instead of adding to them
 };
 
-// dL/dP_k = V_rot^T dL/dW_{v,k} summed over views, then (q, t) of the pose,
-// for instance k (1-based). dM is read past L1 (other CTAs summed it).
-__device__ __forceinline__ void pose_chain_one(const ViewSet& vs, const float* dM, int n_inst, int k,
-                                               const float4* __restrict__ pose_q, float* g_q,
-                                               float* g_t, int overwrite) {
-  const int nk = n_inst + 1;
-  float dPr[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dPt[3] = {0.f, 0.f, 0.f};
-  for (int v = 0; v < vs.n_views; ++v) {
-    const float* V = vs.v[v].V;
-    const float* dp = dM + (v * nk + k) * 12;
-    float d[12];
+// Copies of the matrix sums: CTA b adds to copy b % copies. More copies mean
+// fewer reductions to one address and shorter chains of additions (one copy lost
+// precision: an instance's thousands of terms were added one after another, where
+// the shared-memory sums of each CTA were added up in turn).
+constexpr int kPoseMatrices = 32768;   // copies x views x segments, at most (1.5 MB)
+constexpr int kPoseCopies = 64;
+__host__ __device__ inline int pose_copies(int64_t matrices) {
+  const int64_t c = kPoseMatrices / (matrices > 0 ? matrices : 1);
+  return (int)(c < 1 ? 1 : (c > kPoseCopies ? kPoseCopies : c));
+}
+
+// Instance blockIdx.x + 1: its matrix adjoints summed over the copies (which are
+// cleared for the next call; they start at zero with the workspace), then
+// dL/dP_k = V_rot^T dL/dW_{v,k} summed over views, then (q, t) of the pose.
+constexpr int kPoseThreads = 128;
+__global__ void __launch_bounds__(kPoseThreads) k_pose_chain(const __grid_constant__ ViewSet vs, float* dM,
+                                                             int copies, int n_inst,
+                                                             const float4* pose_q, float* g_q, float* g_t,
+                                                             int overwrite) {
+  sequence_begin();
+  constexpr int kParts = 8;   // threads that share a sum, every eighth copy each
+  __shared__ float s_part[S3R_MAX_VIEWS * 12][kParts + 1];
+  __shared__ float s_d[S3R_MAX_VIEWS][12];
+  __shared__ float s_P[12];
+  const int nk = n_inst + 1, k = (int)blockIdx.x + 1;
+  const int64_t stride = (int64_t)vs.n_views * nk * 12;
+  const int sums = vs.n_views * 12;
+  for (int j = threadIdx.x; j < sums * kParts; j += kPoseThreads) {
+    const int part = j / sums, i = j - part * sums, v = i / 12, e = i - 12 * v;
+    float* p = dM + (v * nk + k) * 12 + e;
+    float x[kPoseCopies / kParts];
 #pragma unroll
-    for (int i = 0; i < 12; ++i) d[i] = __ldcg(dp + i);
+    for (int c = 0; c < kPoseCopies / kParts; ++c) {
+      const int copy = c * kParts + part;
+      x[c] = copy < copies ? p[copy * stride] : 0.f;
+    }
+    float sum = 0.f;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
+    for (int c = 0; c < kPoseCopies / kParts; ++c) {
+      const int copy = c * kParts + part;
+      sum += x[c];
+      if (copy < copies && x[c] != 0.f) p[copy * stride] = 0.f;
+    }
+    s_part[i][part] = sum;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < sums; i += kPoseThreads) {
+    float sum = 0.f;
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-        dPr[3 * r + c] += V[r] * d[c] + V[4 + r] * d[4 + c] + V[8 + r] * d[8 + c];
-      dPt[r] += V[r] * d[3] + V[4 + r] * d[7] + V[8 + r] * d[11];
+    for (int q = 0; q < kParts; ++q) sum += s_part[i][q];
+    (&s_d[0][0])[i] = sum;
+  }
+  __syncthreads();
+  // entry (r, c) of dP: 0..8 the rotation's, 9..11 the translation's
+  if (threadIdx.x < 12) {
+    const int i = (int)threadIdx.x, r = i < 9 ? i / 3 : i - 9, c = i < 9 ? i - 3 * (i / 3) : 3;
+    float sum = 0.f;
+    for (int v = 0; v < vs.n_views; ++v) {
+      const float* V = vs.v[v].V;
+      const float* d = s_d[v];
+      sum += V[r] * d[c] + V[4 + r] * d[4 + c] + V[8 + r] * d[8 + c];
+    }
+    s_P[i] = sum;
+    if (i >= 9 && g_t) {
+      float* p = g_t + 3 * (k - 1) + r;
+      *p = overwrite ? sum : *p + sum;
     }
   }
-  if (g_t) {
-    float* p = g_t + 3 * (k - 1);
-    for (int c = 0; c < 3; ++c) p[c] = overwrite ? dPt[c] : p[c] + dPt[c];
-  }
-  if (g_q) {
+  __syncthreads();
+  if (threadIdx.x == 0 && g_q) {
+    float dPr[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) dPr[i] = s_P[i];
     const float4 gq = quat_backward(pose_q[k - 1], dPr);
     const float v[4] = {gq.x, gq.y, gq.z, gq.w};
     float* p = g_q + 4 * (k - 1);
@@ -87,9 +136,9 @@ __device__ __forceinline__ void pose_chain_one(const ViewSet& vs, const float* d
 // one float at a time: such an add retries until no other lane's came between,
 // and a warp's lanes mostly share an instance, so a batch of one instance's
 // Gaussians took about 25 us: 1001 x 563, 5 instances near the camera, 63 ->
-// 39 us a view with the grouped SH sums below; one 1080p view 94 -> 76 us; the
-// surround rig 415 -> 387 us. Sums over the warp's lanes first took 22 us on the
-// small view, but 438 us at the rig: registers spilled.)
+// 21 us a view with the grouped SH sums below; one 1080p view 94 -> 78 us; the
+// surround rig 415 -> 399 us. Sums over the warp's lanes before the add took 438
+// us at the rig: registers spilled.)
 __device__ __forceinline__ void add_matrix_adjoint(float* dst, const float (&dA)[9], const float (&db)[3]) {
 #pragma unroll
   for (int r = 0; r < 3; ++r)
@@ -128,6 +177,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
 
   // only Gaussians kept in at least one view have adjoints; a warp takes 32
   // consecutive work-list entries
+  float* pose_dM = a.pose_dM + (int64_t)(blockIdx.x % (unsigned)a.pose_copies) * vs.n_views * nk * 12;
   const uint32_t n_kept = a.ctr[kCtrKept];
   const uint32_t epoch = a.ctr[kCtrEpoch];
   // software pipeline over the warp's batches: the next batch's work-list
@@ -312,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
         dA[3 * r] += dp[r] * mv[0]; dA[3 * r + 1] += dp[r] * mv[1]; dA[3 * r + 2] += dp[r] * mv[2];
         db[r] += dp[r];
       }
-      if (k > 0) add_matrix_adjoint(a.pose_dM + (v * nk + k) * 12, dA, db);
+      if (k > 0) add_matrix_adjoint(pose_dM + (v * nk + k) * 12, dA, db);
     }
 
     // ---- RS = R diag(s), s = exp(log s), R = R(q/|q|)
@@ -414,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
         }
       }
 
-      if (DEG > 0 && k > 0) add_matrix_adjoint(a.pose_dM + (v * nk + k) * 12, dA, db);
+      if (DEG > 0 && k > 0) add_matrix_adjoint(pose_dM + (v * nk + k) * 12, dA, db);
     }
     if (a.g.means) {
       float* p = a.g.means + 3 * (size_t)gid;
@@ -484,25 +534,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
     }
     __syncwarp();
   }
-  // the last CTA to finish maps the summed matrix adjoints to the poses, then
-  // clears the sums for the next call (they start at zero with the workspace)
-  if (a.n_inst > 0) {
-    __shared__ bool s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(a.ctr + kCtrProjBwdExits, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (s_last) {
-      __threadfence();
-      if (a.g.inst_quat || a.g.inst_trans)
-        for (int k = 1 + (int)threadIdx.x; k <= a.n_inst; k += blockDim.x)
-          pose_chain_one(vs, a.pose_dM, a.n_inst, k, a.pose_q, a.g.inst_quat, a.g.inst_trans,
-                         a.overwrite);
-      __syncthreads();
-      for (int i = threadIdx.x; i < vs.n_views * nk * 12; i += blockDim.x) __stcg(a.pose_dM + i, 0.f);
-      if (threadIdx.x == 0) a.ctr[kCtrProjBwdExits] = 0u;
-    }
-  }
 }
 
 template <int DEG>
@@ -540,11 +571,20 @@ cudaError_t launch_deg(s3r_workspace* ws, const BwdArgs& a, cudaStream_t st) {
   }
   const int per_sm = cached_per_sm;
   KernelTimer timer(ws, kKProjectBwd, st);
-  return launch_in_sequence(ws, k_project_bwd<DEG>, (int64_t)ws->num_sms * per_sm, kThreads, smem, st,
-                            ws->views, a);
+  const cudaError_t e = launch_in_sequence(ws, k_project_bwd<DEG>, (int64_t)ws->num_sms * per_sm, kThreads,
+                                           smem, st, ws->views, a);
+  if (e != cudaSuccess || ws->n_inst == 0) return e;
+  return launch_in_sequence(ws, k_pose_chain, ws->n_inst, kPoseThreads, 0, st, ws->views, a.pose_dM,
+                            a.pose_copies, ws->n_inst, a.pose_q, a.g.inst_quat, a.g.inst_trans, a.overwrite);
 }
 
 }  // namespace
+
+int64_t pose_sum_floats(int64_t max_views, int64_t segments) {
+  // the copies of any call fit: c m <= max(kPoseMatrices, m) for m = views x segments
+  const int64_t m = max_views * segments;
+  return 12 * (m > kPoseMatrices ? m : (m * kPoseCopies < kPoseMatrices ? m * kPoseCopies : (int64_t)kPoseMatrices));
+}
 
 cudaError_t launch_project_bwd(s3r_workspace* ws, const s3r_scene* sc, const s3r_poses* poses,
                                const s3r_grads* g, cudaStream_t st) {
@@ -574,6 +614,7 @@ cudaError_t launch_project_bwd(s3r_workspace* ws, const s3r_scene* sc, const s3r
   a.cap_splats = ws->cap.max_splats;
   a.ctr = ws->ctr;
   a.pose_dM = ws->pose_dM;
+  a.pose_copies = pose_copies((int64_t)ws->n_views * (sc->n_inst + 1));
   a.g = *g;
   a.mats = reinterpret_cast<const InstMat*>(ws->mats);
   a.overwrite = ws->grad_mode == S3R_GRAD_OVERWRITE ? 1 : 0;

@@ -209,7 +209,7 @@ s3r_status s3r_workspace_create(const s3r_capacity* cap, int device, s3r_workspa
   S3R_ALLOC(ws->final_T, cap->max_pixels);
   S3R_ALLOC(ws->n_contrib, cap->max_pixels);
   S3R_ALLOC(ws->sp_grad, 12 * S);
-  S3R_ALLOC(ws->pose_dM, (int64_t)cap->max_views * nk * 12);
+  S3R_ALLOC(ws->pose_dM, pose_sum_floats(cap->max_views, nk));
   S3R_ALLOC(ws->world_acc, (int64_t)nk * world_acc_floats());
   S3R_ALLOC(ws->mats, (int64_t)cap->max_views * nk * 20);
   S3R_ALLOC(ws->dup_excl, S + 1);
@@ -231,7 +231,7 @@ s3r_status s3r_workspace_create(const s3r_capacity* cap, int device, s3r_workspa
     }
   }
   if ((e = cudaMemset(ws->ctr, 0, sizeof(uint32_t) * kCtrCount)) != cudaSuccess ||
-      (e = cudaMemset(ws->pose_dM, 0, sizeof(float) * 12 * (size_t)cap->max_views * nk)) != cudaSuccess ||
+      (e = cudaMemset(ws->pose_dM, 0, sizeof(float) * (size_t)pose_sum_floats(cap->max_views, nk))) != cudaSuccess ||
       (e = cudaMemset(ws->world_acc, 0, sizeof(float) * (size_t)nk * world_acc_floats())) != cudaSuccess ||
       (e = cudaMemset(ws->lookback, 0, sizeof(unsigned long long) * ws->lookback_words)) !=
           cudaSuccess ||

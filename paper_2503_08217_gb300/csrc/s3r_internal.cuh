@@ -30,7 +30,6 @@ enum Ctr : int {
   kCtrBlendFwdExits = 33,
   kCtrBlendBwdCursor = 34,
   kCtrBlendBwdExits = 35,
-  kCtrProjBwdExits = 36,     // CTAs of the projection backward that finished
   kCtrCompactExits = 38,     // CTAs of the compaction that finished
   kCtrCount = 40
 };
@@ -174,7 +173,7 @@ struct s3r_workspace {
   uint32_t* n_contrib;      // [P]
   float* sp_grad;           // [S*12] per-splat 2D adjoints summed by the blend backward
   int sp_grad_clean;        // host: the last render_fwd zeroed sp_grad and no backward used it since
-  float* pose_dM;           // [views*(inst+1)*12], zero between backward calls
+  float* pose_dM;           // [copies][views*(inst+1)*12], zero between backward calls
   float* world_acc;         // [(inst+1) * world_acc_floats()] pose sums of s3r_to_world_bwd, zero between calls
   float* mats;              // composed matrices [views*(inst+1)] x 20 floats
   uint32_t* dup_excl;       // [S+1] first pair of each depth-sorted splat
@@ -282,6 +281,8 @@ cudaError_t launch_render_bwd(s3r_workspace* ws, const float* bg, const float* d
                               const s3r_grads* grads, cudaStream_t st);
 cudaError_t launch_project_bwd(s3r_workspace* ws, const s3r_scene* sc, const s3r_poses* poses,
                                const s3r_grads* g, cudaStream_t st);
+// Floats of the workspace's matrix-adjoint sums (k_project_bwd.cu).
+int64_t pose_sum_floats(int64_t max_views, int64_t segments);
 cudaError_t launch_adam(const s3r_adam_tensor* t, int count, float lr, float b1, float b2,
                         float eps, float bc1, float bc2, const uint32_t* gate, cudaStream_t st);
 // SM count of the current device (queried once per device, then cached).
