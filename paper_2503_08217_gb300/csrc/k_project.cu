@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kThreads, S3R_PROJECT_MASK_BLOCKS) k_project_m
     uint32_t fmask = 0, kmask = 0, gid = 0;
     if (active) {
       gid = a.selected[j];
-      const int k = segment_of(s_off, a.n_inst, gid);
+      const int k = segment_of<true>(s_off, a.n_inst, gid);
       const float mu[3] = {a.means[3 * (size_t)gid], a.means[3 * (size_t)gid + 1],
                            a.means[3 * (size_t)gid + 2]};
       const float s0 = __expf(a.log_scales[3 * (size_t)gid]);

@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_bwd(const __grid_consta
 #pragma unroll
     for (int i = 0; i < K * 3; ++i) g_sh[i] = 0.f;
     if (kmask) {
-    const int k = segment_of(s_off, a.n_inst, gid);
+    const int k = segment_of<true>(s_off, a.n_inst, gid);
     uint32_t s = s0;
 
     const float sc[3] = {__expf(ls[0]), __expf(ls[1]), __expf(ls[2])};

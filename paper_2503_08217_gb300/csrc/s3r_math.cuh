@@ -68,8 +68,14 @@ __device__ __forceinline__ void cam_pos(const InstMat& M, const float d[3], floa
 }
 
 // Segment (0 = static, k = instance k) of Gaussian `gid` from the offsets.
+// kStaticFirst: most Gaussians are static and a warp's ids ascend, so most warps
+// need one comparison instead of the search (the mask kernel at 8M Gaussians, 80
+// instances: one view 134 -> 129 us, seven 390 -> 375 us; the projection backward
+// of the seven 397 -> 389 us; no gain where kept splats are written).
+template <bool kStaticFirst = false>
 __device__ __forceinline__ int segment_of(const uint32_t* off, int n_inst, uint32_t gid) {
-  int lo = 0, hi = n_inst + 1;  // off[lo] <= gid < off[hi]
+  if (kStaticFirst && gid < off[1]) return 0;
+  int lo = kStaticFirst ? 1 : 0, hi = n_inst + 1;  // off[lo] <= gid < off[hi]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (off[mid] <= gid) lo = mid; else hi = mid;
