@@ -9,9 +9,9 @@
 // K); the splats are then expanded into (tile, splat) pairs in depth order,
 // and the one or two tile-digit passes finish the sort. Every pass is a
 // single-pass "onesweep" kernel: persistent CTAs take tiles of kSortTileKeys
-// keys (3840 by default) from an atomic counter, rank digits with eight warp
-// ballots per key (faster here than match.any, which queues on the
-// address-divergence unit), get each digit's global offset from a
+// keys (3840 by default) from an atomic counter, rank digits through shared
+// memory or with warp ballots (match.any queues on the address-divergence
+// unit), get each digit's global offset from a
 // precomputed histogram plus a decoupled look-back over tiles, reorder the
 // tile in shared memory and write it out coalesced.
 #include "s3r_internal.cuh"
@@ -28,6 +28,8 @@ constexpr int kWarpKeys = kSortItems * 32;   // keys per warp per tile
 #endif
 constexpr int kSortLookback = S3R_SORT_LOOKBACK;
 static_assert(kSortLookback >= 1 && kSortLookback <= 64, "look-back batch of 1..64 words");
+
+constexpr int kShortBits = 6;   // see k_onesweep
 
 struct PassArgs {
   const uint32_t* keys_in;
@@ -89,14 +91,27 @@ __device__ __forceinline__ void load_tile(const PassArgs& a, int64_t n, int64_t 
   }
 }
 
-// One LSD pass. Per tile: rank the digits (eight warp ballots per key),
-// publish the tile's digit counts for the look-back, reorder the tile by digit
-// in shared memory, take the next tile and start its loads, then walk the
-// look-back for the global offsets (thread d for digit d, eight predecessors
-// per round trip) while those loads are in flight, and write the reordered
-// tile out.
+// One LSD pass. Per tile: rank the digits, publish the tile's digit counts for
+// the look-back, reorder the tile by digit in shared memory, take the next tile
+// and start its loads, then walk the look-back for the global offsets (thread d
+// for digit d, eight predecessors per round trip) while those loads are in
+// flight, and write the reordered tile out.
+//
+// The pass is bound by its instructions (177 per 32 keys, most of them on the
+// ALU pipe, when digits were ranked with eight ballots a key). kSpread ranks
+// through shared memory instead: one OR a key finds the lanes with the same
+// digit. That is for digits that spread over many values, since lanes with equal
+// digits wait for each other there: the three low digits of the depth and the
+// tile digits (23.9M pairs of a seven-camera rig, in a captured step: 0.188 and
+// 0.180 -> 0.162 and 0.168 ms a pass; 4.8M splats: 0.046 -> 0.040). The depth's top digit, its exponent, has few values
+// and keeps the ballots (0.043 ms, 0.042 either way), and so does a tile digit
+// of up to kShortBits bits, which takes a ballot a bit (11.2M pairs, the upper
+// six bits of 9,600 tiles: 0.078 ms against 0.090 through shared memory).
+template <int kBits, bool kSpread>
 __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(PassArgs a) {
   sequence_begin();
+  constexpr uint32_t kMask = (1u << kBits) - 1u;
+  static_assert(kSortTileKeys >= kWarps * kRadix, "the reorder buffers hold a word per warp and digit");
   __shared__ uint32_t s_keys[kSortTileKeys];
   __shared__ uint32_t s_vals[kSortTileKeys];
   __shared__ uint32_t s_cnt[kWarps][kRadix];   // per-warp digit counts -> exclusive offsets
@@ -124,23 +139,57 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
     for (int i = lane; i < kRadix; i += 32) s_cnt[warp][i] = 0;
     __syncwarp();
     uint32_t rank[kSortItems];
+    if constexpr (kSpread) {
+      // peers with the same digit: each lane sets its bit in the digit's word, two
+      // rounds at a time (the reorder buffers hold the words); the first of the
+      // peers adds their number to the warp's count
+      uint32_t* const words[2] = {s_keys + warp * kRadix, s_vals + warp * kRadix};
+      uint32_t before[kSortItems];
+      for (int i = lane; i < kRadix; i += 32) words[0][i] = words[1][i] = 0u;
+      __syncwarp();
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-      // peers with the same digit: the AND over the digit's eight bits of the
-      // ballot or its complement (padding keys rank last within digit 255)
-      const uint32_t d = (key[r] >> a.shift) & (kRadix - 1);
-      uint32_t peers = 0xffffffffu;
+      for (int r = 0; r < kSortItems; r += 2) {
 #pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-        peers &= bit ? bal : ~bal;
+        for (int q = 0; q < 2 && r + q < kSortItems; ++q)
+          atomicOr(words[q] + ((key[r + q] >> a.shift) & kMask), 1u << lane);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 2 && r + q < kSortItems; ++q)
+          rank[r + q] = words[q][(key[r + q] >> a.shift) & kMask];
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 2 && r + q < kSortItems; ++q) {
+          const uint32_t d = (key[r + q] >> a.shift) & kMask;
+          before[r + q] = 0u;
+          if ((rank[r + q] & lt) == 0) {
+            words[q][d] = 0u;
+            before[r + q] = atomicAdd(&s_cnt[warp][d], (uint32_t)__popc(rank[r + q]));
+          }
+          __syncwarp();
+        }
       }
-      const uint32_t before = s_cnt[warp][d];
-      rank[r] = before + __popc(peers & lt);
-      __syncwarp();
-      if ((peers & lt) == 0) s_cnt[warp][d] = before + __popc(peers);
-      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < kSortItems; ++r)
+        rank[r] = __shfl_sync(0xffffffffu, before[r], __ffs(rank[r]) - 1) + __popc(rank[r] & lt);
+    } else {
+#pragma unroll
+      for (int r = 0; r < kSortItems; ++r) {
+        // peers with the same digit: the AND over the digit's bits of the
+        // ballot or its complement
+        const uint32_t d = (key[r] >> a.shift) & kMask;
+        uint32_t peers = 0xffffffffu;
+#pragma unroll
+        for (int b = 0; b < kBits; ++b) {
+          const bool bit = (d >> b) & 1u;
+          const uint32_t bal = __ballot_sync(0xffffffffu, bit);
+          peers &= bit ? bal : ~bal;
+        }
+        const uint32_t before = s_cnt[warp][d];
+        rank[r] = before + __popc(peers & lt);
+        __syncwarp();
+        if ((peers & lt) == 0) s_cnt[warp][d] = before + __popc(peers);
+        __syncwarp();
+      }
     }
     __syncthreads();
 
@@ -163,7 +212,7 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
 #pragma unroll
     for (int r = 0; r < kSortItems; ++r) {
       if (base + r * 32 + lane < n) {
-        const uint32_t d = (key[r] >> a.shift) & (kRadix - 1);
+        const uint32_t d = (key[r] >> a.shift) & kMask;
         const uint32_t pos = s_loc[d] + s_cnt[warp][d] + rank[r];
         s_keys[pos] = key[r];
         s_vals[pos] = val[r];
@@ -185,7 +234,7 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
     const int tile_n = (int)min((int64_t)kSortTileKeys, n - tile * kSortTileKeys);
     for (int i = threadIdx.x; i < tile_n; i += kSortThreads) {
       const uint32_t k = s_keys[i];
-      const uint32_t dst = s_dst[(k >> a.shift) & (kRadix - 1)] + (uint32_t)i;
+      const uint32_t dst = s_dst[(k >> a.shift) & kMask] + (uint32_t)i;
       __stcs(a.keys_out + dst, k);
       __stcs(a.vals_out + dst, s_vals[i]);
     }
@@ -222,8 +271,9 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
 //                rectangle) and a 32-byte record for the expansion: the splat
 //                id, the tile id of the rectangle's corner, grid and
 //                rectangle widths, rectangle height, and its rows: the first
-//                kInlineRows in the record, the others 4 bytes each in a row
-//                table (offsets from a warp-aggregated bump counter; the warp
+//                kInlineRows in the record, the others 8 bytes each in a row
+//                table (columns, and the tiles of the splat before the
+//                row, which the expansion files its markers by; offsets from a warp-aggregated bump counter; the warp
 //                computes a tall splat's rows together, one per lane), so
 //                that the expansion reads most splats' rows without a
 //                dependent load. A splat that no longer fits the table
@@ -909,7 +959,10 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
   cudaError_t e;
   // occupancy is queried once (outside any graph capture: the first call)
   static thread_local int sweep_per_sm = 0, dup_per_sm = 0, exp_per_sm = 0;
-  if (!sweep_per_sm) sweep_per_sm = per_sm_for((const void*)k_onesweep, kSortThreads);
+  if (!sweep_per_sm)
+    sweep_per_sm = min(per_sm_for((const void*)k_onesweep<kRadixBits, true>, kSortThreads),
+                       min(per_sm_for((const void*)k_onesweep<kRadixBits, false>, kSortThreads),
+                           per_sm_for((const void*)k_onesweep<kShortBits, false>, kSortThreads)));
   if (!dup_per_sm) dup_per_sm = per_sm_for((const void*)k_dup_scan, kDupThreads);
   if (!exp_per_sm) exp_per_sm = per_sm_for((const void*)k_dup_expand, kDupThreads);
   const int g_sweep = ws->num_sms * sweep_per_sm;
@@ -928,7 +981,8 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     a.lookback = ws->lookback;
     a.stage = kStageDepth0 + p;
     KernelTimer timer(ws, kKDepth0 + p, st);
-    e = launch_in_sequence(ws, k_onesweep, g_sweep, kSortThreads, 0, st, a);
+    e = launch_in_sequence(ws, p < 3 ? k_onesweep<kRadixBits, true> : k_onesweep<kRadixBits, false>, g_sweep,
+                           kSortThreads, 0, st, a);
     if (e != cudaSuccess) return e;
   }
   ws->depth_final = 0;
@@ -1000,7 +1054,10 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
     a.lookback = ws->lookback;
     a.stage = kStageTile0 + p;
     KernelTimer timer(ws, kKTile0 + p, st);
-    e = launch_in_sequence(ws, k_onesweep, g_sweep, kSortThreads, 0, st, a);
+    // tile ids are below total_tiles, so the last digit may have few bits (see k_onesweep)
+    const bool few = ((ws->views.total_tiles - 1) >> (8 * p)) < (1 << kShortBits);
+    e = launch_in_sequence(ws, few ? k_onesweep<kShortBits, false> : k_onesweep<kRadixBits, true>, g_sweep,
+                           kSortThreads, 0, st, a);
     if (e != cudaSuccess) return e;
   }
   ws->dup_final = ws->tile_passes & 1;

@@ -323,6 +323,25 @@ def test_expansion_of_tall_and_wide_splats(count, width, height):
         _stage_isolated_sort(res, cams)
 
 
+@pytest.mark.parametrize("width,height", [(32, 16), (128, 128), (80, 208), (2048, 2048), (2064, 2048)])
+def test_sort_at_short_tile_digits(width, height):
+    """2, 64, 65, 16,384 and 16,512 tiles: both sides of the lines (6 bits of the
+    first and of the second digit) between the two ways of ranking a digit."""
+    import gpu_helpers
+    from test_gpu_parity import _stage_isolated_sort
+    rng = np.random.default_rng(53)
+    count = 600
+    g = scenegen.generate("fd", seed=3, n_static=count, n_inst=0, n_steps=2)
+    g.means[:] = rng.uniform((-3, -3, 3), (3, 3, 9), (count, 3))
+    g.log_scales[:] = np.log(rng.uniform(0.01, 0.1, (count, 3)))
+    cams = [make_camera(width, height, 0.5 * max(width, height), (0.0, 0.0, 0.0), 0.0)]
+    g = scenegen.with_cameras(g, [cams, cams])
+    r = gpu_helpers.Renderer(g.n, 0, cams, max_duplicates=1 << 20)
+    res = _step(g, cams, oracle.vis_reset(count)[0], None, step=0, renderer=r)
+    assert res["counts"]["n_duplicates"] > count // 4
+    _stage_isolated_sort(res, cams)
+
+
 @pytest.mark.parametrize("n_inst", [40, 260])
 def test_pose_sums_with_many_instances(tiny, n_inst):
     """Empty instances after the scene's own: fewer copies of the pose sums (64
