@@ -284,10 +284,9 @@ def kernel_models(counts, scene, n_kept_gaussians: int, n_pixels: int, tiles: in
         # offsets and records and writes the pairs
         "splat_tiles": ("hbm", S * (4 + 32) + S * (4 + 32)),
         "duplicate": ("hbm", S * (4 + 4)),
-        "duplicate_expand": ("hbm", S * (4 + 32) + K * 8),   # + tile-digit histograms (on chip)
-        # per tile: its range and class slot out (the binary searches' reads
-        # are cached); the forward's contributor bits cleared
-        "tile_ranges": ("hbm", tiles * (8 + 4) + K / 8 * 2),
+        "duplicate_expand": ("hbm", S * (4 + 32) + K * 8 + K / 8 * 2),   # pairs, and contributor bits cleared
+        # per tile: its range and class slot out (the searches' reads are cached)
+        "tile_ranges": ("hbm", tiles * (8 + 4)),
         # overwrite mode: kept rows written once (no read), the splat adjoints read
         "project_bwd": ("hbm", n_kept_gaussians * (12 + geo + kk + (geo + kk)) + S * 48),
         # FP32 operations per evaluated (pixel, splat) pair, counted in the code
@@ -539,9 +538,10 @@ def run_ours(args, rank, world, local):
                 roof.update(fused_zeroing_bytes=table[dom]["zero_bytes"],
                             frac_alu_plus_hbm=table[dom]["frac_alu_plus_hbm"])
     # the timed kernels, plus untimed ones of ours: the L1 loss and the zeroing
-    # of its output and, for the conventional pipeline, the world transform and
-    # its backward (two launches)
-    launches_per_step = len(kmean) + 2 + (3 if args.conventional else 0)
+    # of its output, the poses' launch inside the projection backward's time and,
+    # for the conventional pipeline (whose render has no instances), the world
+    # transform and its backward (two launches)
+    launches_per_step = len(kmean) + 2 + (3 if args.conventional else int(scene.n_inst > 0))
 
     # --- plain per-view comparator: the same library, one camera per call, eager
     plain = None
@@ -889,7 +889,7 @@ def run_ode(args):
         "data": "synthetic", "forward_ms": round(ms_fwd, 4),
         "config": {"workload": "ode: " + WORKLOADS["ode"][3], "instances": K, "output_times": T,
                    "substeps": S, "rk4_steps_per_instance": steps, "hidden": H, "embed_dim": D},
-        "roofline": {"bound": "latency (one warp per instance, sequential steps)",
+        "roofline": {"bound": "latency (one CTA per instance, sequential steps)",
                      "achieved_gops": round(ops / (ms_both / 1e3) / 1e9, 1),
                      "alu_peak_gops": round(peak / 1e9, 1),
                      "frac": round(ops / (ms_both / 1e3) / peak, 4)},

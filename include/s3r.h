@@ -394,7 +394,8 @@ s3r_status s3r_kernel_times(s3r_workspace* ws, float* ms, int32_t n);
  *               return S3R_ERR_TIMEOUT, which is only known on the device).
  * The look-back scratch is a fixed array in the library's device image
  * (about 128 KB, held by every GPU that loads the library until the process
- * exits); every call shares it and clears the part it uses on entry, so
+ * exits); every call shares it and clears its counters on entry (the look-back
+ * words are tagged with a call counter kept there), so
  * calls that overlap on the GPU (e.g. on two streams at once) race and must
  * be serialised by the caller. The first call on a device looks up the
  * array's device address and the device's SM count (once per device); make
@@ -485,7 +486,8 @@ s3r_status s3r_set_epoch(s3r_workspace* ws, uint32_t epoch, void* stream);
  *         "tile_ranges" uint2[tiles]; "final_T" float[pixels];
  *         "n_contrib" u32[pixels]; "splat_grads" float[n_splats*12]
  *         (du, dv, dA, dB, dC, dopacity, dr, dg, db, 0, 0, 0);
- *         "pose_grad_matrix" float[n_views*(n_inst+1)*12] dL/dW_{t,i}.
+ *         "pose_grad_matrix" float[copies][n_views*(n_inst+1)*12], the sums of
+ *         dL/dW_{t,i} during a backward (zero between calls).
  * Returns NULL for an unknown name. */
 const void* s3r_debug_buffer(const s3r_workspace* ws, const char* name);
 
