@@ -370,7 +370,6 @@ struct StaticScratch {
 
 static __device__ __align__(256) StaticScratch g_static_scratch;
 
-constexpr int kMaxDevices = 64;
 const ViewSet g_no_views = {};   // the selection composes no matrices
 std::mutex g_static_mutex;
 StaticScratch* g_static_ptr[kMaxDevices] = {};

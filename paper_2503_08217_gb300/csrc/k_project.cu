@@ -470,15 +470,19 @@ cudaError_t launch_deg(s3r_workspace* ws, const ProjArgs& a, cudaStream_t st) {
   const size_t smem_splats = sizeof(float) * kWarps * ShStage<DEG>::kWords + smem;
   // occupancy is queried once (the first, eager call), so that a launch
   // inside CUDA-graph capture issues nothing but the kernels
-  static thread_local int per_mask = 0, per_splats = 0, per_scan = 0;
+  // (the writer's shared-memory limit is a property of the function on one
+  // device, so its figures are kept by device)
+  static thread_local int per_mask = 0, per_splats_on[kMaxDevices] = {}, per_scan = 0;
+  int& per_splats = per_splats_on[ws->device % kMaxDevices];
+  cudaError_t e;
   if (!per_mask) per_mask = occupancy(k_project_mask, smem);
   if (!per_splats) {
-    cudaFuncSetAttribute(k_project_splats<DEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(float) * kWarps * ShStage<DEG>::kWords + 16 * 1024));
+    e = cudaFuncSetAttribute(k_project_splats<DEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(float) * kWarps * ShStage<DEG>::kWords + 16 * 1024));
+    if (e != cudaSuccess) return e;
     per_splats = occupancy(k_project_splats<DEG>, smem_splats);
   }
   if (!per_scan) per_scan = occupancy(k_splat_scan, 0);
-  cudaError_t e;
   {
     KernelTimer timer(ws, kKProject, st);
     e = launch_in_sequence(ws, k_project_mask, (int64_t)ws->num_sms * per_mask, kThreads, smem, st,

@@ -541,35 +541,38 @@ cudaError_t launch_deg(s3r_workspace* ws, const BwdArgs& a, cudaStream_t st) {
   const int nk = ws->n_inst + 1;
   const size_t smem = sizeof(float) * kWarps * ShStage<DEG>::kWords +
                       sizeof(uint32_t) * (nk + 1) + 16;
-  // The dynamic shared-memory limit is a property of the function, shared by all
-  // threads, and the size depends on the scene: it is raised once to the most
-  // the device allows, so that no thread's scene lowers it under another's.
-  static thread_local int most = 0;
-  static thread_local size_t cached_smem = 0;
-  static thread_local int cached_per_sm = 0;
-  if (!most) {
-    int dev = 0, optin = 0;
+  // The dynamic shared-memory limit is a property of the function on one device,
+  // shared by all threads, and the size depends on the scene: on each device it
+  // is raised once to the most the device allows, so that no thread's scene
+  // lowers it under another's.
+  struct Shape {
+    int most = 0, per_sm = 0;
+    size_t smem = 0;   // what per_sm is for
+  };
+  static thread_local Shape shapes[kMaxDevices];
+  Shape& on = shapes[ws->device % kMaxDevices];
+  if (!on.most) {
+    int optin = 0;
     cudaFuncAttributes fa;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ws->device);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_project_bwd<DEG>);
     if (e != cudaSuccess) return e;
     const int room = optin - (int)fa.sharedSizeBytes;
     e = cudaFuncSetAttribute(k_project_bwd<DEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
     if (e != cudaSuccess) return e;
-    most = room;
+    on.most = room;
   }
-  if (smem > (size_t)most) return cudaErrorInvalidValue;
-  if (smem != cached_smem) {
+  if (smem > (size_t)on.most) return cudaErrorInvalidValue;
+  if (smem != on.smem) {
     int per_sm = 0;
     const cudaError_t e =
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_project_bwd<DEG>, kThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    cached_smem = smem;
-    cached_per_sm = per_sm;
+    on.smem = smem;
+    on.per_sm = per_sm;
   }
-  const int per_sm = cached_per_sm;
+  const int per_sm = on.per_sm;
   KernelTimer timer(ws, kKProjectBwd, st);
   const cudaError_t e = launch_in_sequence(ws, k_project_bwd<DEG>, (int64_t)ws->num_sms * per_sm, kThreads,
                                            smem, st, ws->views, a);

@@ -127,7 +127,6 @@ s3r_status set_last_error(s3r_status st, const char* msg) {
 }
 
 int sm_count() {
-  constexpr int kMaxDevices = 64;
   static std::atomic<int> cache[kMaxDevices];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;

@@ -285,6 +285,8 @@ cudaError_t launch_project_bwd(s3r_workspace* ws, const s3r_scene* sc, const s3r
 int64_t pose_sum_floats(int64_t max_views, int64_t segments);
 cudaError_t launch_adam(const s3r_adam_tensor* t, int count, float lr, float b1, float b2,
                         float eps, float bc1, float bc2, const uint32_t* gate, cudaStream_t st);
+// Entries of the tables kept by device ordinal.
+constexpr int kMaxDevices = 64;
 // SM count of the current device (queried once per device, then cached).
 int sm_count();
 // Zero `words` 32-bit words at a 16-byte aligned device address with a
