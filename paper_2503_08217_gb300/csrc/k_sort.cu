@@ -111,9 +111,11 @@ template <int kBits, bool kSpread>
 __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(PassArgs a) {
   sequence_begin();
   constexpr uint32_t kMask = (1u << kBits) - 1u;
-  static_assert(kSortTileKeys >= kWarps * kRadix, "the reorder buffers hold a word per warp and digit");
-  __shared__ uint32_t s_keys[kSortTileKeys];
-  __shared__ uint32_t s_vals[kSortTileKeys];
+  // the reorder buffers, which also hold a word per warp and digit while kSpread
+  // ranks (more than a tile of fewer than eight keys per thread has)
+  constexpr int kBuffer = kSpread && kSortTileKeys < kWarps * kRadix ? kWarps * kRadix : kSortTileKeys;
+  __shared__ uint32_t s_keys[kBuffer];
+  __shared__ uint32_t s_vals[kBuffer];
   __shared__ uint32_t s_cnt[kWarps][kRadix];   // per-warp digit counts -> exclusive offsets
   __shared__ uint32_t s_gbase[kRadix];         // exclusive scan of the global histogram
   __shared__ uint32_t s_loc[kRadix];           // tile-local start of each digit

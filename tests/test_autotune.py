@@ -213,3 +213,14 @@ def test_report_carries_each_trials_clocks_and_the_second_timing():
     assert "| 1 | A=2 | 5.500 | 1.100 | 1800 / 2070 MHz, sw_power_cap |" in text
     assert "timed again in a fresh process: 5.050 ms / step (+1.00 %" in text
     assert autotune.clock_note({"clocks": {"sm_mhz": None, "reasons": ["no samples"]}}) == "not sampled"
+
+
+@pytest.mark.skipif(not HAVE_NVCC, reason="nvcc is needed to compile")
+@pytest.mark.parametrize("items", [1, 2, 7, 8])
+def test_radix_tiles_below_the_candidates_compile(items):
+    """The source takes 1 to 18 keys per thread, also where a tile is smaller
+    than the words the digits are ranked with."""
+    r = subprocess.run([libbuild.nvcc(), "-arch=sm_103a", "-O3", "-std=c++17", "-I" + libbuild.INCLUDE,
+                        "-DS3R_ARCH=103", "-cubin", "-o", os.devnull, f"-DS3R_SORT_ITEMS={items}",
+                        os.path.join(libbuild.CSRC, "k_sort.cu")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr

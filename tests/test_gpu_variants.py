@@ -65,3 +65,8 @@ def test_off_default_launch_shapes_pass_parity(defines):
                          ids=["two_scan_ctas", "unpacked_tile_inputs"])
 def test_untuned_shapes_pass_parity(defines):
     _parity_with(defines)
+
+
+def test_small_radix_tiles_pass_parity():
+    """Tiles of fewer keys than the words the digits are ranked with."""
+    _parity_with({"S3R_SORT_ITEMS": 3})
