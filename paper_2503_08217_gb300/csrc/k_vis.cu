@@ -4,7 +4,8 @@
 //   RESET    v = (-1, 1), l = (1, -1): visible at all times, empty life.
 // A plain streaming pass. Where both arrays are 16-byte aligned a thread takes
 // four pairs of Gaussians (one 128-bit access per pair and array, the four
-// loads issued together); a sub-range that starts at an odd index has only
+// loads issued together; RECORD stores 64 bits where only one of a pair is seen);
+// a sub-range that starts at an odd index has only
 // 8-byte alignment and takes one Gaussian per access.
 #include "s3r_internal.cuh"
 
@@ -62,15 +63,14 @@ __global__ void __launch_bounds__(kVisThreads) k_vis_pairs(int64_t n, float t,
     } else if (MODE == S3R_VIS_FINALIZE) {
       vis[p] = make_float4(l[q].x - 0.1f, l[q].y + 0.1f, l[q].z - 0.1f, l[q].w + 0.1f);
     } else {
-      if (seen[q] & 1u) {
-        l[q].x = fminf(l[q].x, t);
-        l[q].y = fmaxf(l[q].y, t);
-      }
-      if (seen[q] & 2u) {
-        l[q].z = fminf(l[q].z, t);
-        l[q].w = fmaxf(l[q].w, t);
-      }
-      life[p] = l[q];
+      // a Gaussian whose bit is clear is never written: calls on other streams
+      // may record disjoint masks of the same array at the same time
+      const float2 a = make_float2(fminf(l[q].x, t), fmaxf(l[q].y, t));
+      const float2 b = make_float2(fminf(l[q].z, t), fmaxf(l[q].w, t));
+      if (seen[q] == 3u)
+        life[p] = make_float4(a.x, a.y, b.x, b.y);
+      else
+        reinterpret_cast<float2*>(life)[2 * p + (seen[q] >> 1)] = (seen[q] & 1u) ? a : b;
     }
   }
   if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)   // the last Gaussian of an odd count
