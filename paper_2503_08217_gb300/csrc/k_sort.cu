@@ -770,10 +770,19 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
     const uint32_t q0 = a.dup_chunk[chunk], q1 = a.dup_chunk[chunk + 1];
     for (uint32_t qb = q0 + warp * 32; qb <= q1; qb += kDupThreads) {
       const uint32_t q = qb + lane;
-      uint32_t o = 0, o0 = 0, corner = 0, gx = 0, w = 0, h = 0, off = 0, sp = 0;
+      uint32_t o = c.O1, o0 = c.O1, corner = 0, gx = 0, w = 0, h = 0, off = 0, sp = 0;
+      uint4 d = make_uint4(0u, 0u, 0u, 0u), e = d;
       if (q <= q1) {
-        const uint4 d = a.dup_meta[2 * (size_t)q], e = a.dup_meta[2 * (size_t)q + 1];
+        d = a.dup_meta[2 * (size_t)q];
+        e = a.dup_meta[2 * (size_t)q + 1];
         o0 = o = a.dup_excl[q];
+      }
+      // The last chunk's map ends at the last splat, and splats without a pair
+      // (too faint to reach a tile) may follow the last one that has some: past
+      // the chunk's outputs nothing is left to file. (A view of 82,000 pairs with
+      // 960,000 faint splats behind them took 2.3 ms here without this.)
+      if (__shfl_sync(0xffffffffu, o0, 0) >= c.O1) break;
+      if (q <= q1) {
         sp = d.x;
         corner = d.y;
         gx = d.z & 0xffffu;
