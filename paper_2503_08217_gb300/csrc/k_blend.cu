@@ -2,7 +2,8 @@
 // adjoint.
 //
 // Forward: one CTA of two warps per tile, each warp a 16x8 band, four pixels
-// per lane, the two of a column evaluated as one packed f32x2 pair. The
+// per lane, the two of a column evaluated as one packed f32x2 pair (on small
+// images four warps, each a 16x4 band, two pixels per lane). The
 // tile's front-to-back splat list is consumed in batches (64 by default) staged in
 // shared memory (uv, base-2 conic, opacity, rgb as duplicated pairs, and the
 // box where the splat can reach alpha >= 1/255); per 32 splats a warp ballots which of
@@ -172,21 +173,26 @@ __device__ __forceinline__ void queue_exit(const TileQueue& q) {
 
 // The forward's form of the same queue: the CTA's first warp finds the class
 // starts with one load per lane (not 33 dependent ones) and a position's class
-// with one compare per lane, and where the launch has a CTA for every item, CTA
-// i takes item i and the cursor stays untouched.
+// with one compare per lane. A CTA's first position is its own number, the cursor
+// counts those after the grid: an SM's CTAs start together, and where they drew
+// their first positions from the cursor, the longest lists met on one SM. Where
+// the launch has a CTA for every tile it is direct: CTA i takes tile i, then the zeroing chunks grid - 1 - i, + grid, ...,
+// so that the chunks go to the CTAs without a tile or with the shortest ones
+// first and the cursor stays untouched. (Chunks spread among the tiles, as the
+// cursor hands them out, held the last tiles back until others had ended: 1,196
+// tiles of a view of 381,000 splats 86 us, 57 us without any zeroing.)
 struct QueueState {
-  uint32_t pending;   // warp 0: the position taken, one item ahead
+  uint32_t pending;   // warp 0: the position taken, one item ahead; direct: the
+                      // tile, from gridDim.x on that plus the next chunk
   bool direct;
 };
 __device__ __forceinline__ void fwd_queue_init(const BlendArgs& a, uint32_t* s_cstart,
                                                uint32_t n_chunks, QueueState& st) {
   static_assert(kTileClasses == 33, "a lane per class, and one more");
-  const bool many = (uint32_t)a.tiles > gridDim.x;
   st.pending = blockIdx.x;
-  st.direct = !many;
+  st.direct = (uint32_t)a.tiles <= gridDim.x;
   if (threadIdx.x < 32) {
     const uint32_t lane = threadIdx.x;
-    if (many && lane == 0) st.pending = atomicAdd(a.fwd_queue.cursor, 1u);
     const uint32_t c = a.class_cnt[lane], c_last = a.class_cnt[kTileClasses - 1];
     uint32_t incl = c;
 #pragma unroll
@@ -202,31 +208,39 @@ __device__ __forceinline__ void fwd_queue_init(const BlendArgs& a, uint32_t* s_c
     }
   }
   __syncthreads();
-  if (!many && s_cstart[kTileClasses] + n_chunks > gridDim.x) {   // block-uniform
-    st.direct = false;
-    if (threadIdx.x == 0) st.pending = atomicAdd(a.fwd_queue.cursor, 1u);
-  }
 }
 
 __device__ __forceinline__ int fwd_queue_next(const BlendArgs& a, const uint32_t* s_cstart,
                                               int* s_tile, QueueState& st) {
   if (threadIdx.x < 32) {
-    const uint32_t i = __shfl_sync(0xffffffffu, st.pending, 0);
-    const uint64_t T = s_cstart[kTileClasses], C = s_cstart[kTileClasses + 1];
-    const uint64_t P = T + C;
+    uint32_t i = __shfl_sync(0xffffffffu, st.pending, 0);
+    const uint32_t T = s_cstart[kTileClasses], C = s_cstart[kTileClasses + 1];
     int t = -1;
-    if (i < P) {
-      if (threadIdx.x == 0) st.pending = st.direct ? 0xffffffffu : atomicAdd(a.fwd_queue.cursor, 1u);
+    uint32_t ti = 0xffffffffu;   // the tile's place in the queue, if the item is one
+    if (st.direct) {
+      if (i < gridDim.x) {
+        if (i < T) ti = i;
+        i = 2u * gridDim.x - 1u - i;   // the first chunk, which is the item where there is no tile
+        st.pending = i;
+      }
+      if (ti == 0xffffffffu && i - gridDim.x < C) {
+        t = -2 - (int)(i - gridDim.x);
+        st.pending = i + gridDim.x;
+      }
+    } else if (i < (uint64_t)T + C) {
+      if (threadIdx.x == 0) st.pending = gridDim.x + atomicAdd(a.fwd_queue.cursor, 1u);
+      const uint64_t P = (uint64_t)T + C;
       const uint64_t cb = C ? (uint64_t)i * C / P : 0u;              // chunks before position i
       const uint64_t cb1 = C ? ((uint64_t)i + 1u) * C / P : 0u;
-      if (cb1 > cb) {
+      if (cb1 > cb)
         t = -2 - (int)cb;
-      } else {
-        const uint32_t ti = (uint32_t)(i - cb);                          // tiles before position i
-        // class starts ascend: the class is the number of later starts at or below ti
-        const int c = __popc(__ballot_sync(0xffffffffu, ti >= s_cstart[threadIdx.x + 1]));
-        t = (int)a.class_list[(size_t)c * a.tiles + (ti - s_cstart[c])];
-      }
+      else
+        ti = (uint32_t)(i - cb);                                       // tiles before position i
+    }
+    if (ti != 0xffffffffu) {
+      // class starts ascend: the class is the number of later starts at or below ti
+      const int c = __popc(__ballot_sync(0xffffffffu, ti >= s_cstart[threadIdx.x + 1]));
+      t = (int)a.class_list[(size_t)c * a.tiles + (ti - s_cstart[c])];
     }
     if (threadIdx.x == 0) *s_tile = t;
   }
@@ -553,10 +567,9 @@ __device__ __forceinline__ bool all_stopped(const float (&floor_)[kPix]) {
 // few registers more than 48 end the spills.
 //
 // kWarpsT: warps per tile. Two (16x8 bands, four pixels per lane) share a
-// splat's loads and loop between the most pixels. Where the image has so few
-// tiles that all of them are resident at once, the time is that of the longest
-// list walked by one pair of warps, and four (16x4 bands, two pixels per lane)
-// walk it faster: see launch_render_fwd for the line and both sides' times. The
+// splat's loads and loop between the most pixels. On a small image the time is
+// that of the longest list walked by one pair of warps, and four (16x4 bands, two
+// pixels per lane) walk it faster: see launch_fwd for the line and its times. The
 // contributor bits stay those of the backward's 16x8 bands, two warps adding
 // to each.
 template <bool kCount, int kWarpsT>
@@ -839,7 +852,7 @@ __device__ __forceinline__ void bwd_init(BwdPixel& q, const BlendArgs& a, const 
 
 // One splat of the backward's walk (see above) over a lane's two packed
 // pixel pairs: updates T and Bd, returns the lane's shares of the nine sums in
-// g. kClamp as for fwd_splat, per splat.
+// g. kClamp as for fwd_eval, per splat.
 //
 // A pixel that does not take the splat gets G = 0, hence alpha 0: 1 / (1 - 0) is
 // exactly 1, so T, the weight and every sum are left unchanged by the same
@@ -1214,12 +1227,34 @@ int blend_blocks_per_sm(K kernel, int threads, int* cache) {
   return *cache;
 }
 
+// CTAs of a forward launch: as many as are resident at once.
 template <bool kCount, int kWarpsT>
-cudaError_t launch_fwd(s3r_workspace* ws, const BlendArgs& a, cudaStream_t st) {
+int fwd_grid(const s3r_workspace* ws) {
   static thread_local int per_sm = 0;
-  constexpr int kThreadsT = 32 * kWarpsT;
-  const int g = ws->num_sms * blend_blocks_per_sm(k_blend_fwd<kCount, kWarpsT>, kThreadsT, &per_sm);
-  return launch_in_sequence(ws, k_blend_fwd<kCount, kWarpsT>, g, kThreadsT, 0, st, ws->views, a);
+  return ws->num_sms * blend_blocks_per_sm(k_blend_fwd<kCount, kWarpsT>, 32 * kWarpsT, &per_sm);
+}
+
+// Four warps per tile where every tile has a resident CTA of them (1,368 tiles on
+// 152 SMs): the longest list decides, and they walk it faster. With more tiles than
+// that the work of all lists decides, unless the scene has so few Gaussians that
+// most tiles are nearly empty: four up to twice as many tiles then. Times of the
+// kernel with two and with four warps, us, by tiles (corridors; Gaussians, views):
+//                 240        920        1,296      1,674      2,405      2,800
+//   300,000, 1   125 / 80    80 / 59    74 / 61    74 / 84    80 / 117   88 / 119
+//   1M, 1         94 / 61    68 / 53    68 / 57    70 / 84    76 / 108   90 / 113
+//   4M, 1         74 / 49    55 / 53    59 / 59    63 / 96    76 / 104  100 / 113
+//   20,000, 1    141 / 96    84 / 55    66 / 45    68 / 51    61 / 47    61 / 49
+// and by Gaussians at 2,442 to 2,508 tiles: 20,000 over 80 m 68 / 53, three views
+// 111 / 74; 40,000 over 60 m 66 / 59; 70,000 84 / 88, three views 102 / 92; 120,000
+// 74 / 113, three views 90 / 131.
+constexpr int64_t kSparseGaussians = 80000;
+template <bool kCount>
+cudaError_t launch_fwd(s3r_workspace* ws, const BlendArgs& a, cudaStream_t st) {
+  const int g4 = fwd_grid<kCount, 4>(ws), g2 = fwd_grid<kCount, 2>(ws);
+  const int tiles = ws->views.total_tiles;
+  if (tiles <= g4 || (tiles <= g2 && ws->n <= kSparseGaussians))
+    return launch_in_sequence(ws, k_blend_fwd<kCount, 4>, g4, 128, 0, st, ws->views, a);
+  return launch_in_sequence(ws, k_blend_fwd<kCount, 2>, g2, 64, 0, st, ws->views, a);
 }
 
 cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cudaStream_t st) {
@@ -1233,13 +1268,8 @@ cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cu
     if ((e = cudaMemsetAsync(a.pairs, 0, 2 * sizeof(unsigned long long), st)) != cudaSuccess) return e;
   }
   // the contributor bits were cleared by the sort's pair expansion
-  // four warps per tile where every tile is resident at once with two (see k_blend_fwd)
-  const bool few = ws->views.total_tiles <= ws->num_sms * S3R_BLEND_FWD_BLOCKS;
   KernelTimer timer(ws, kKBlendFwd, st);
-  if (ws->counting)
-    e = few ? launch_fwd<true, 4>(ws, a, st) : launch_fwd<true, 2>(ws, a, st);
-  else
-    e = few ? launch_fwd<false, 4>(ws, a, st) : launch_fwd<false, 2>(ws, a, st);
+  e = ws->counting ? launch_fwd<true>(ws, a, st) : launch_fwd<false>(ws, a, st);
   ws->sp_grad_clean = 1;
   return e;
 }
