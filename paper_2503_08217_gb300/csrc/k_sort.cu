@@ -107,6 +107,20 @@ __device__ __forceinline__ void load_tile(const PassArgs& a, int64_t n, int64_t 
 // and keeps the ballots (0.043 ms, 0.042 either way), and so does a tile digit
 // of up to kShortBits bits, which takes a ballot a bit (11.2M pairs, the upper
 // six bits of 9,600 tiles: 0.078 ms against 0.090 through shared memory).
+//
+// Where many keys share a digit, a spread pass takes longer than ballots do: all
+// keys alike (a flat wall seen head on, 5M splats) 0.049 ms against 0.045, a tile
+// digit of which one value has 0.6 of the keys (12.8M pairs) 0.114 against 0.102.
+// A choice by the histogram's largest count inside the kernel mended those passes
+// but made every other one 6 to 9 % longer (the rig's tile passes 0.185 -> 0.201
+// and 0.192 -> 0.209 ms), so there is none: the passes of such a view together
+// took 0.39 to 0.41 ms both ways.
+
+// Place of a digit's word: digits that are multiples of 32, as the low depth digit
+// is far from the origin, where depths are coarse, fall into different banks (four
+// such values, 5M splats: 0.058 ms in one bank, 0.043 so; ballots 0.045).
+__device__ __forceinline__ uint32_t word_of(uint32_t d) { return d ^ (d >> 5); }
+
 template <int kBits, bool kSpread>
 __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(PassArgs a) {
   sequence_begin();
@@ -153,18 +167,18 @@ __global__ void __launch_bounds__(kSortThreads, S3R_SORT_BLOCKS) k_onesweep(Pass
       for (int r = 0; r < kSortItems; r += 2) {
 #pragma unroll
         for (int q = 0; q < 2 && r + q < kSortItems; ++q)
-          atomicOr(words[q] + ((key[r + q] >> a.shift) & kMask), 1u << lane);
+          atomicOr(words[q] + word_of((key[r + q] >> a.shift) & kMask), 1u << lane);
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 2 && r + q < kSortItems; ++q)
-          rank[r + q] = words[q][(key[r + q] >> a.shift) & kMask];
+          rank[r + q] = words[q][word_of((key[r + q] >> a.shift) & kMask)];
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 2 && r + q < kSortItems; ++q) {
           const uint32_t d = (key[r + q] >> a.shift) & kMask;
           before[r + q] = 0u;
           if ((rank[r + q] & lt) == 0) {
-            words[q][d] = 0u;
+            words[q][word_of(d)] = 0u;
             before[r + q] = atomicAdd(&s_cnt[warp][d], (uint32_t)__popc(rank[r + q]));
           }
           __syncwarp();

@@ -98,3 +98,24 @@ def test_forward_queue_forms_agree():
                 if a.size:
                     np.testing.assert_allclose(res["grads"][k], a, rtol=1e-4, atol=5e-5 * max(np.abs(a).max(), 1e-30),
                                                err_msg=k)
+
+
+@pytest.mark.parametrize("values", [1, 4, 1000])
+def test_sort_of_coarse_depths(values):
+    """Depths of few values, their low digits multiples of 64 (a flat wall, and a
+    scene far from the origin): equal depths keep the splats' order."""
+    import gpu_helpers
+    from test_gpu_parity import _stage_isolated_sort
+    count = 9000
+    rng = np.random.default_rng(values)
+    g = scenegen.generate("fd", seed=7, n_static=count, n_inst=0, n_steps=2)
+    z = (16.0 + rng.integers(0, values, count) * 2.0 ** -13).astype(np.float32)
+    g.means[:] = np.stack([rng.uniform(-0.9, 0.9, count) * z, rng.uniform(-0.9, 0.9, count) * z, z], 1)
+    g.log_scales[:] = np.log(0.05)
+    cams = [make_camera(480, 480, 240.0, (0.0, 0.0, 0.0), 0.0)]
+    g = scenegen.with_cameras(g, [cams, cams])
+    res = gpu_helpers.gpu_step(g, 0, cams, oracle.vis_reset(count)[0])
+    assert res["counts"]["n_splats"] > count // 2
+    depth = np.unique(res["rgb_d"][:, 3].view(np.uint32))
+    assert depth.size <= values and not (depth & 63).any()
+    _stage_isolated_sort(res, cams)
