@@ -74,6 +74,10 @@ struct GradZero {
   int sh_floats;                   // 3 (K + 1)^2
 };
 
+// Which of a call's forward launches works: always, where the longest list decides
+// the time, or where the work of all lists does (see long_list_decides).
+enum Pick { kPickAlways = 0, kPickLongList, kPickEvenLists };
+
 struct BlendArgs {
   const uint2* ranges;
   const uint32_t* class_cnt;    // [kTileClasses] tiles per class
@@ -91,7 +95,8 @@ struct BlendArgs {
   uint32_t* n_contrib;
   float* sp_grad;         // [S*12]: zeroed by the forward (chunks in its queue), summed by the backward
   const uint32_t* ctr;
-  int64_t cap_splats;
+  int64_t cap_splats, cap_dups;
+  int pick;               // forward only: which of two launches of a call works (see launch_fwd)
   unsigned long long* pairs;     // counting mode: list pairs the forward walked
   unsigned long long* eval_fwd;  // counting mode: pairs the forward evaluated
   unsigned long long* eval_bwd;  // counting mode: pairs the backward evaluated
@@ -186,7 +191,18 @@ struct QueueState {
                       // tile, from gridDim.x on that plus the next chunk
   bool direct;
 };
-__device__ __forceinline__ void fwd_queue_init(const BlendArgs& a, uint32_t* s_cstart,
+// Whether the forward's time is that of the tile with the longest list, from the
+// first class that has tiles: that list at least three times the mean, and so few
+// pairs that the SMs do not wait for issue slots (launch_fwd has the times).
+constexpr uint32_t kFewPairs = 300000, kLongList = 3;
+__device__ __forceinline__ bool long_list_decides(const BlendArgs& a, uint32_t first_class) {
+  const uint32_t pairs = (uint32_t)min((int64_t)a.ctr[kCtrDups], a.cap_dups);
+  const uint32_t longest = 0x80000000u >> first_class;   // and less than twice that
+  return pairs <= kFewPairs && (uint64_t)longest * (uint32_t)a.tiles >= (uint64_t)kLongList * pairs;
+}
+
+// False: this launch is not the one that works.
+__device__ __forceinline__ bool fwd_queue_init(const BlendArgs& a, uint32_t* s_cstart, int* s_works,
                                                uint32_t n_chunks, QueueState& st) {
   static_assert(kTileClasses == 33, "a lane per class, and one more");
   st.pending = blockIdx.x;
@@ -206,8 +222,14 @@ __device__ __forceinline__ void fwd_queue_init(const BlendArgs& a, uint32_t* s_c
       s_cstart[kTileClasses] = incl + c_last;
       s_cstart[kTileClasses + 1] = n_chunks;
     }
+    if (a.pick != kPickAlways) {
+      const uint32_t listed = __ballot_sync(0xffffffffu, c > 0u);
+      const bool decides = listed && long_list_decides(a, (uint32_t)__ffs(listed) - 1u);
+      if (lane == 0) *s_works = decides == (a.pick == kPickLongList);
+    }
   }
   __syncthreads();
+  return a.pick == kPickAlways || *s_works;
 }
 
 __device__ __forceinline__ int fwd_queue_next(const BlendArgs& a, const uint32_t* s_cstart,
@@ -587,9 +609,9 @@ __global__ void __launch_bounds__(32 * kWarpsT, S3R_BLEND_FWD_BLOCKS * kBandWarp
   __shared__ float2 s_u[kBatchFwd];    // u u
   __shared__ float4 s_box[kBatchFwd];
   __shared__ uint32_t s_cstart[kTileClasses + 2];
-  __shared__ int s_tile;
+  __shared__ int s_tile, s_works;
   QueueState queue;
-  fwd_queue_init(a, s_cstart, splat_grad_chunks(a), queue);
+  if (!fwd_queue_init(a, s_cstart, &s_works, splat_grad_chunks(a), queue)) return;
   for (;;) {
     const int tile = fwd_queue_next(a, s_cstart, &s_tile, queue);
     if (tile == -1) break;
@@ -1195,6 +1217,8 @@ static BlendArgs make_args(s3r_workspace* ws) {
   a.fwd_queue = TileQueue{ws->ctr + kCtrBlendFwdCursor, ws->ctr + kCtrBlendFwdExits};
   a.ctr = ws->ctr;
   a.cap_splats = ws->cap.max_splats;
+  a.cap_dups = ws->cap.max_duplicates;
+  a.pick = kPickAlways;
   a.bwd_queue = TileQueue{ws->ctr + kCtrBlendBwdCursor, ws->ctr + kCtrBlendBwdExits};
   a.zero = GradZero{nullptr, 0, {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}, 0};
   a.sorted_splats = ws->dup_val[ws->dup_final];
@@ -1235,26 +1259,44 @@ int fwd_grid(const s3r_workspace* ws) {
 }
 
 // Four warps per tile where every tile has a resident CTA of them (1,368 tiles on
-// 152 SMs): the longest list decides, and they walk it faster. With more tiles than
-// that the work of all lists decides, unless the scene has so few Gaussians that
-// most tiles are nearly empty: four up to twice as many tiles then. Times of the
-// kernel with two and with four warps, us, by tiles (corridors; Gaussians, views):
-//                 240        920        1,296      1,674      2,405      2,800
-//   300,000, 1   125 / 80    80 / 59    74 / 61    74 / 84    80 / 117   88 / 119
-//   1M, 1         94 / 61    68 / 53    68 / 57    70 / 84    76 / 108   90 / 113
-//   4M, 1         74 / 49    55 / 53    59 / 59    63 / 96    76 / 104  100 / 113
-//   20,000, 1    141 / 96    84 / 55    66 / 45    68 / 51    61 / 47    61 / 49
-// and by Gaussians at 2,442 to 2,508 tiles: 20,000 over 80 m 68 / 53, three views
-// 111 / 74; 40,000 over 60 m 66 / 59; 70,000 84 / 88, three views 102 / 92; 120,000
-// 74 / 113, three views 90 / 131.
-constexpr int64_t kSparseGaussians = 80000;
+// 152 SMs): they walk the longest list faster. With up to twice as many tiles it is
+// in the lists, which only the device knows, whether one of them or the work of all
+// decides: both forms are launched, and the one that is not to work returns at once
+// (about 2 us). With more tiles still, two warps. Times of the kernel with two and
+// with four warps, us (corridors; by tiles, then with the pairs and the longest list
+// over the mean):
+//   Gaussians        240        920      1,296      1,674      2,405      2,800
+//   300,000     125 / 80    80 / 59    74 / 61    74 / 84   80 / 117   88 / 119
+//   1M           94 / 61    68 / 53    68 / 57    70 / 84   76 / 108   90 / 113
+//   4M           74 / 49    55 / 53    59 / 59    63 / 96   76 / 104  100 / 113
+//   1,500 to 2,700 tiles
+//     109,000 pairs, 56: 205 / 139     173,000, 44: 295 / 170    152,000, 18: 72 / 53
+//     205,000 pairs, 2:   55 / 86      450,000, 3:   80 / 125    380,000, 4:  60 / 90
+//     667,000 pairs, 16:  80 / 123     842,000, 43:  84 / 94     327,000, 8: 102 / 80
+// Of 67 such images drawn at random the rule takes the slower form in 8, by 4 to 43 us;
+// all with two warps took 7 % longer together, all with four 17 %.
+//
+// Only the smallest of these launches overlap their predecessor's end: placed then, a
+// grid that is resident at once ends up unevenly over the SMs, and the longest lists
+// share some. Whole forward, us, overlapped and not: 22,000 Gaussians, 320 x 192 165
+// and 167, 960 x 540 155 and 157; 150,000 at 320 x 192 172 and 176, 640 x 360 168 and
+// 162, 960 x 540 212 and 193; 300,000 at 960 x 540 241 and 209, three views of 576 x
+// 324 295 and 245; 1M at 640 x 360 244 and 225, at 1080p (more tiles than CTAs) equal.
+constexpr int64_t kOverlapBlendGaussians = 50000;
+constexpr int kOverlapBlendTiles = 2;   // per SM
 template <bool kCount>
-cudaError_t launch_fwd(s3r_workspace* ws, const BlendArgs& a, cudaStream_t st) {
+cudaError_t launch_fwd(s3r_workspace* ws, BlendArgs& a, cudaStream_t st) {
   const int g4 = fwd_grid<kCount, 4>(ws), g2 = fwd_grid<kCount, 2>(ws);
   const int tiles = ws->views.total_tiles;
-  if (tiles <= g4 || (tiles <= g2 && ws->n <= kSparseGaussians))
-    return launch_in_sequence(ws, k_blend_fwd<kCount, 4>, g4, 128, 0, st, ws->views, a);
-  return launch_in_sequence(ws, k_blend_fwd<kCount, 2>, g2, 64, 0, st, ws->views, a);
+  const bool by_lists = tiles > g4 && tiles <= g2;
+  const bool overlap = ws->overlap && (ws->n <= kOverlapBlendGaussians || tiles <= kOverlapBlendTiles * ws->num_sms);
+  if (tiles > g4) {
+    a.pick = by_lists ? kPickEvenLists : kPickAlways;
+    const cudaError_t e = launch_overlapping(overlap, k_blend_fwd<kCount, 2>, g2, 64, 0, st, ws->views, a);
+    if (e != cudaSuccess || !by_lists) return e;
+  }
+  a.pick = by_lists ? kPickLongList : kPickAlways;
+  return launch_overlapping(overlap && !by_lists, k_blend_fwd<kCount, 4>, g4, 128, 0, st, ws->views, a);
 }
 
 cudaError_t launch_render_fwd(s3r_workspace* ws, const float* bg, float* out, cudaStream_t st) {

@@ -242,15 +242,18 @@ namespace s3r {
 // their start-up when the predecessor ends. A kernel of the sequence may thus
 // be resident while an earlier one still writes the workspace, so none reads
 // the workspace through the read-only path (__ldg, const __restrict__).
-// The 14 to 19 launches of a call gain 1 to 2 us each: an image of 22,000
-// Gaussians 149 -> 119 us, two 1001 x 563 training steps 1084 -> 993 us, one
-// 1080p view of 1.1M 477 -> 467 us. With 9M Gaussians the waiting blocks cost
-// more than that (1920 x 1280 at full detail 1265 -> 1288 us, surround rig 4862
-// -> 4899 us), so the line lies between the two.
+// The 14 to 19 launches of a call gain 1 to 2 us each, but the waiting blocks cost
+// the larger scenes more than that. Time without overlap over the time with it, one
+// view forward at 640 x 360 and at 1080p: 0.6M Gaussians 1.06 and 1.05, 1.5M 1.01 and
+// 1.03, 2M 1.03 and 1.03, 3M 0.97 and 1.02, 4.5M 0.98 and 0.98, 7M 0.97 and 0.98;
+// with the backward 1.05 and 1.04, 1.01 and 1.01, 2M 1.02 and 1.02, 3M 1.01 and 0.99,
+// 7M 1.00 and 0.99. Seven views of 640 x 360 gain 1 to 6 % at all of these sizes, seven
+// of 1080p are within 0.6 % either way. The forward blend has a narrower rule
+// (launch_fwd).
 constexpr int64_t kOverlapGaussians = 2000000;
 template <typename... P, typename... A>
-cudaError_t launch_in_sequence(const s3r_workspace* ws, void (*kernel)(P...), int64_t grid, int threads,
-                               size_t smem, cudaStream_t st, const A&... args) {
+cudaError_t launch_overlapping(bool overlap, void (*kernel)(P...), int64_t grid, int threads, size_t smem,
+                               cudaStream_t st, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)threads);
@@ -260,8 +263,13 @@ cudaError_t launch_in_sequence(const s3r_workspace* ws, void (*kernel)(P...), in
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = ws->overlap ? 1 : 0;
+  cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_in_sequence(const s3r_workspace* ws, void (*kernel)(P...), int64_t grid, int threads,
+                               size_t smem, cudaStream_t st, const A&... args) {
+  return launch_overlapping(ws->overlap != 0, kernel, grid, threads, smem, st, args...);
 }
 
 // ---- launchers (one translation unit each) ---------------------------------

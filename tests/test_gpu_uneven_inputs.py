@@ -62,19 +62,20 @@ def test_faint_splats_behind_the_last_pair():
     assert ms["duplicate_expand"] <= 10 * ms["duplicate"], ms
 
 
-def test_forward_queue_forms_agree():
-    """One image as 1, 2 and 3 copies: four warps per tile and a CTA for every tile,
-    two warps and a CTA for every tile, and tiles drawn from the cursor, each with
-    more clearing chunks (2,048 splats) than CTAs without a tile. Same pixels and
-    last contributors, gradients in proportion, also in a second step (cursor and
-    splat adjoints are back at zero)."""
+@pytest.mark.parametrize("count,extent", [(300_000, 0.95), (20_000, 0.02)], ids=["even", "long_list"])
+def test_forward_queue_forms_agree(count, extent):
+    """One image as 1, 2 and 3 copies: four warps per tile and a CTA for every tile;
+    the tile counts at which the lists choose between two and four warps (evenly
+    filled tiles, or nearly all splats in a few tiles); two warps and tiles drawn
+    from the cursor. With the even lists there are more clearing chunks (2,048
+    splats) than CTAs without a tile. Same pixels and last contributors, gradients
+    in proportion, also in a second step (cursor and splat adjoints are back at zero)."""
     import gpu_helpers
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    count = 300_000
     rng = np.random.default_rng(67)
     g = scenegen.generate("fd", seed=6, n_static=count, n_inst=0, n_steps=2)
     z = rng.uniform(4, 12, count)
-    g.means[:] = np.stack([rng.uniform(-0.95, 0.95, count) * z, rng.uniform(-0.75, 0.75, count) * z, z], 1)
+    g.means[:] = np.stack([rng.uniform(-extent, extent, count) * z, rng.uniform(-0.8 * extent, 0.8 * extent, count) * z, z], 1)
     g.log_scales[:] = np.log(rng.uniform(0.002, 0.02, (count, 3)))
     rows = 9 * sms // 40                                    # 40 x rows tiles, at most 9 CTAs per SM
     cam = make_camera(640, 16 * rows, 320.0, (0.0, 0.0, 0.0), 0.0)
@@ -88,8 +89,13 @@ def test_forward_queue_forms_agree():
         r = gpu_helpers.Renderer(g.n, 0, cams, max_splats=count * copies, max_duplicates=16 * count)
         for _ in range(2):
             res = gpu_helpers.gpu_step(g, 0, cams, vis, dL=[d / copies] * copies, renderer=r)
-            chunks, tiles = -(-res["counts"]["n_splats"] // 2048), 40 * rows * copies
-            assert chunks > 9 * sms - 40 * rows and (copies > 1) == (tiles > 9 * sms) and (copies > 2) == (tiles > 18 * sms)
+            chunks, tiles, pairs = -(-res["counts"]["n_splats"] // 2048), 40 * rows * copies, res["counts"]["n_duplicates"]
+            assert (copies > 1) == (tiles > 9 * sms) and (copies > 2) == (tiles > 18 * sms)
+            longest = int((res["ranges"][:, 1] - res["ranges"][:, 0]).max())
+            if extent > 0.5:
+                assert chunks > 9 * sms - 40 * rows and pairs > 300_000
+            else:
+                assert pairs < 300_000 and longest * tiles > 6 * pairs
             first = first or res
             for v in range(copies):
                 np.testing.assert_allclose(res["images"][v], first["images"][0], rtol=0, atol=1e-6)
