@@ -81,9 +81,9 @@ void free_all(s3r_workspace* ws) {
     if (p) cudaFree(p);
 }
 
-// Dynamic shared memory the projection kernels need for n_views x segments.
-size_t proj_smem_bytes(int n_views, int n_inst) {
-  return (size_t)n_views * (n_inst + 1) * (80 + 48) + 4 * (size_t)(n_inst + 2) + 16;
+// Bytes of a call's n_views x segments matrices and its instance offsets.
+int64_t matrix_bytes(int n_views, int n_inst) {
+  return (int64_t)n_views * (n_inst + 1) * kMatrixBytes + 4 * ((int64_t)n_inst + 2) + 16;
 }
 
 s3r_status check_scene(const s3r_workspace* ws, const s3r_scene* sc) {
@@ -269,7 +269,7 @@ s3r_status s3r_project(s3r_workspace* ws, const s3r_scene* scene, const s3r_pose
     return fail(S3R_ERR_INVALID, "point_life must be 8-byte aligned");
   if (!std::isfinite(t) || !std::isfinite(lod_threshold))
     return fail(S3R_ERR_INVALID, "t and lod_threshold must be finite");
-  if (proj_smem_bytes(n_views, scene->n_inst) > 200 * 1024)
+  if (matrix_bytes(n_views, scene->n_inst) > kMatrixBudget)
     return fail(S3R_ERR_INVALID, "n_views x (n_inst+1) = %d x %d exceeds the shared-memory budget",
                 n_views, scene->n_inst + 1);
   ViewSet vs;

@@ -289,6 +289,10 @@ cudaError_t launch_render_bwd(s3r_workspace* ws, const float* bg, const float* d
                               const s3r_grads* grads, cudaStream_t st);
 cudaError_t launch_project_bwd(s3r_workspace* ws, const s3r_scene* sc, const s3r_poses* poses,
                                const s3r_grads* g, cudaStream_t st);
+// Composed matrices (views x segments) a call takes at most: 128 bytes each within
+// the 200 KB that s3r_project allows them.
+constexpr int64_t kMatrixBytes = 80 + 48, kMatrixBudget = 200 * 1024;
+constexpr int64_t kMaxMatrices = kMatrixBudget / kMatrixBytes;
 // Floats of the workspace's matrix-adjoint sums (k_project_bwd.cu).
 int64_t pose_sum_floats(int64_t max_views, int64_t segments);
 cudaError_t launch_adam(const s3r_adam_tensor* t, int count, float lr, float b1, float b2,

@@ -125,3 +125,53 @@ def test_sort_of_coarse_depths(values):
     depth = np.unique(res["rgb_d"][:, 3].view(np.uint32))
     assert depth.size <= values and not (depth & 63).any()
     _stage_isolated_sort(res, cams)
+
+
+def test_pose_adjoint_of_a_large_instance_keeps_its_precision():
+    """One instance of 400,000 Gaussians beside 259 empty ones (1,566 matrices, near
+    the most a call takes): its pose adjoint against the FP64 sum of those of the
+    same Gaussians as 100 instances with the same pose. Partial sums per CTA gave a
+    mean error of 5.2e-7 of the largest entry, 20 partial sums 1.3e-6; the bound is
+    one and a half times the former."""
+    from paper_2503_08217_gb300.render import DeviceScene, Renderer
+    static, count, parts = 2000, 400_000, 100
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(71)
+    n = static + count
+    uni = lambda lo, hi, *s: torch.empty(s, device="cuda").uniform_(lo, hi, generator=gen)        # noqa: E731
+    means = torch.stack([uni(-20, 20, n), uni(-2, 15, n), uni(0, 60, n)], 1)
+    means[static:] = torch.stack([uni(-8, 8, count), uni(-3, 3, count), uni(-8, 8, count)], 1)
+    quats = torch.empty(n, 4, device="cuda").normal_(generator=gen)
+    scene = DeviceScene(means=means.contiguous(), log_scales=torch.full((n, 3), -3.5, device="cuda"),
+                        quats=(quats / quats.norm(dim=1, keepdim=True)).contiguous(),
+                        opacity_logits=torch.empty(n, device="cuda").normal_(generator=gen),
+                        sh=torch.empty(n, 4, 3, device="cuda").normal_(0, 0.3, generator=gen),
+                        inst_offsets=torch.zeros(3, dtype=torch.int64, device="cuda"), sh_degree=1)
+    cams = [make_camera(640, 360, 320.0, (0.0, 0.0, 30.0), 2 * np.pi * k / 6) for k in range(6)]
+    pixels = 6 * 640 * 360
+    dL = torch.empty(3 * pixels, device="cuda").normal_(0, 1.0 / pixels, generator=gen)
+    window = torch.tensor([-1.0, 1.0], device="cuda").repeat(n, 1).contiguous()
+    bg = torch.zeros(3, device="cuda")
+
+    def adjoint(offsets, n_inst):
+        scene.inst_offsets = torch.tensor(offsets, dtype=torch.int64, device="cuda")
+        quat = torch.tensor([[0.999, 0.0, 0.0447, 0.0]], device="cuda").repeat(n_inst, 1).contiguous()
+        trans = torch.tensor([[0.3, 1.0, 30.2]], device="cuda").repeat(n_inst, 1).contiguous()
+        r = Renderer(n, n_inst, cams, max_splats=6 * n, max_duplicates=1 << 24)
+        r.forward(scene, quat, trans, cams, 0.0, window, None, 0.5, bg)
+        grads = {k: torch.zeros_like(t) for k, t in zip(("means", "log_scales", "quats", "opacity_logits", "sh",
+                                                         "inst_quat", "inst_trans"), scene.params() + [quat, trans])}
+        r.backward(scene, quat, trans, bg, dL, grads)
+        r.sync_status()
+        g = torch.cat([grads["inst_quat"], grads["inst_trans"]], 1).double().cpu().numpy()
+        assert r.counts()["n_splats"] > count // 2
+        return g
+
+    split = [0] + [static + k * (count // parts) for k in range(parts)] + [n]
+    want = np.mean([adjoint(split, parts).sum(0) for _ in range(3)], 0)
+    errors = []
+    for _ in range(6):
+        g = adjoint([0, static] + [n] * 260, 260)
+        assert not g[1:].any()
+        errors.append(np.abs(g[0] - want).max() / np.abs(want).max())
+    assert np.mean(errors) <= 8e-7, errors
