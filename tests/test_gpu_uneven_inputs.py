@@ -175,3 +175,40 @@ def test_pose_adjoint_of_a_large_instance_keeps_its_precision():
         assert not g[1:].any()
         errors.append(np.abs(g[0] - want).max() / np.abs(want).max())
     assert np.mean(errors) <= 8e-7, errors
+
+
+@pytest.mark.parametrize("n_inst", [1, 3, 4, 5, 4001])
+def test_world_adjoints_of_tiny_instances(n_inst):
+    """Instances of 0 to 2 Gaussians, whole and broken groups of the four that a CTA
+    maps to poses: dt is the sum of the rows' adjoints, equal poses with equal rows
+    get equal adjoints, empty instances zero, and a second call repeats the first
+    (the sums were cleared)."""
+    from paper_2503_08217_gb300 import binding
+    from paper_2503_08217_gb300.render import Renderer
+    rng = np.random.default_rng(n_inst)
+    sizes = np.arange(n_inst) % 3
+    off = np.r_[0, 7, 7 + np.cumsum(sizes)].astype(np.int64)
+    n = int(off[-1])
+    cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()   # noqa: E731
+    f32 = lambda *s: rng.standard_normal(s).astype(np.float32)        # noqa: E731
+    means, quats, sh = cu(f32(n, 3)), cu(f32(n, 4)), cu(f32(n, 16, 3))
+    pq, pt = cu(np.tile(f32(1, 4), (n_inst, 1))), cu(f32(n_inst, 3))
+    log_scales, logits, offsets = cu(f32(n, 3)), cu(f32(n)), cu(off)      # held: the scene keeps addresses only
+    cs = binding.make_scene(means, log_scales, quats, logits, sh, offsets, 3)
+    poses = binding.make_poses(pq, pt)
+    r = Renderer(n, n_inst, [make_camera(16, 16, 14.0, (0.0, 0.0, 0.0), 0.0)])
+    up = {"means": f32(n, 3), "quats": f32(n, 4), "sh": f32(n, 16, 3)}
+    got = []
+    for _ in range(2):
+        g = {k: cu(v) for k, v in up.items()}
+        g["inst_quat"] = torch.full((n_inst, 4), float("nan"), device="cuda")
+        g["inst_trans"] = torch.full((n_inst, 3), float("nan"), device="cuda")
+        r.ws.to_world_bwd(cs, poses, g)
+        got.append({k: v.cpu().numpy() for k, v in g.items()})
+    want = np.array([up["means"][off[k + 1]:off[k + 2]].sum(0) for k in range(n_inst)])
+    np.testing.assert_allclose(got[0]["inst_trans"], want, rtol=0, atol=1e-6)
+    assert not got[0]["inst_quat"][sizes == 0].any()
+    if (sizes > 0).any():
+        assert np.abs(got[0]["inst_quat"][sizes > 0]).max(axis=1).min() > 0
+    for k in got[0]:
+        np.testing.assert_array_equal(got[0][k], got[1][k])
