@@ -100,7 +100,7 @@ struct BlendArgs {
   unsigned long long* pairs;     // counting mode: list pairs the forward walked
   unsigned long long* eval_fwd;  // counting mode: pairs the forward evaluated
   unsigned long long* eval_bwd;  // counting mode: pairs the backward evaluated
-  uint32_t* contrib;          // [bands][contrib_words]: pair blended into >= 1 pixel of the band
+  uint32_t* contrib;          // [kBlendBands][contrib_words]: pair blended into >= 1 pixel of the band
   int64_t contrib_words;
 };
 
@@ -407,7 +407,7 @@ __device__ __forceinline__ float4 alpha_box(const float2 xy, const float4 co) {
 // workload), while the per-splat work of a warp (the footprint ballot, the
 // loop and the loads; in the backward the nine-value warp sum, its dominant
 // cost) is shared by 2 * (4 / kBandWarps) pixels per lane.
-constexpr int kBandWarps = 2;
+constexpr int kBandWarps = kBlendBands;
 constexpr int kBandThreads = 32 * kBandWarps;
 constexpr int kBandRows = 4 / kBandWarps;       // pixel rows per lane and column
 constexpr int kBandPix = 2 * kBandRows;         // pixels per lane

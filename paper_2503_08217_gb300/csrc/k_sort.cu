@@ -401,9 +401,6 @@ __device__ __forceinline__ uint2 row_span(const Region& g, uint32_t r, uint32_t 
 struct DupArgs {
   uint32_t* hist;        // tile-digit histograms of the radix passes that follow
   int tile_passes;
-  const uint32_t* sorted_splats;
-  const uint2* sp_rect;
-  const uint8_t* sp_view;
   const uint32_t* sp_cnt;      // [S] tiles each splat reaches, by depth position
   const uint2* row_spans;      // per row of a rectangle: first | end << 16 (columns), and the
                                // splat's tiles before the row
@@ -417,9 +414,8 @@ struct DupArgs {
   int64_t cap_splats, cap_dups;
   uint32_t* ctr;
   unsigned long long* lookback;
-  uint32_t* contrib;       // [bands][contrib_words] the forward's contributor bits, cleared here
+  uint32_t* contrib;       // [kBlendBands][contrib_words] the forward's contributor bits, cleared here
   int64_t contrib_words;
-  int bands;
 };
 
 constexpr int kTilesThreads = 256;
@@ -897,7 +893,7 @@ __global__ void __launch_bounds__(kDupThreads) k_dup_expand(DupArgs a) {
     // many words as there are pairs, where clearing them for the whole pair
     // capacity in the tile-range launch (a few CTAs on small images) took most
     // of that launch
-    for (int b = 0; b < a.bands; ++b)
+    for (int b = 0; b < kBlendBands; ++b)
       for (uint32_t i = threadIdx.x; i < (n_here + 31u) / 32u; i += kDupThreads)
         a.contrib[b * a.contrib_words + c.O0 / 32u + i] = 0u;
     __syncthreads();   // the markers are rewritten by the next chunk
@@ -1013,9 +1009,6 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
   ws->depth_final = 0;
   // expand into (tile, splat) pairs in depth order
   DupArgs d;
-  d.sorted_splats = ws->depth_val[0];
-  d.sp_rect = ws->sp_rect;
-  d.sp_view = ws->sp_view;
   d.sp_cnt = ws->sp_tiles;
   d.row_spans = ws->row_spans;
   d.sp_region = reinterpret_cast<const float4*>(ws->sp_region);
@@ -1032,7 +1025,6 @@ cudaError_t launch_sort(s3r_workspace* ws, cudaStream_t st) {
   d.tile_passes = ws->tile_passes;
   d.contrib = ws->contrib;
   d.contrib_words = ws->contrib_words;
-  d.bands = 2;
   {
     static thread_local int tiles_per_sm = 0;
     if (!tiles_per_sm) tiles_per_sm = per_sm_for((const void*)k_splat_tiles, kTilesThreads);

@@ -220,7 +220,7 @@ s3r_status s3r_workspace_create(const s3r_capacity* cap, int device, s3r_workspa
   S3R_ALLOC(ws->row_spans, ws->rows_cap);
   S3R_ALLOC(ws->dup_chunk, K / kDupChunkMin + 2);
   ws->contrib_words = K / 32 + 2;
-  S3R_ALLOC(ws->contrib, 4 * ws->contrib_words);
+  S3R_ALLOC(ws->contrib, kBlendBands * ws->contrib_words);
 #undef S3R_ALLOC
   for (int i = 0; i < 2 * kKCount; ++i) {
     if ((e = cudaEventCreate(&ws->ev[i])) != cudaSuccess) {

@@ -12,6 +12,11 @@ namespace s3r {
 constexpr int kTile = S3R_TILE;            // 16x16 pixel tiles
 constexpr int kTilePixels = kTile * kTile;
 
+// Bands of 16 / kBlendBands pixel rows that a tile's contributor bits are kept for
+// (and warps per tile of the backward blend): one array of bits each, allocated with
+// the workspace, cleared by the pair expansion, set and read by the blends.
+constexpr int kBlendBands = 2;
+
 // ---- device counters (uint32 slots of ws->ctr) -----------------------------
 enum Ctr : int {
   kCtrSelected = 0,   // Gaussians whose window contains t
@@ -46,7 +51,6 @@ enum Stage : int {
   kStageDup = 2,
   kStageDepth0 = 3,   // 3..6: depth radix passes
   kStageTile0 = 7,    // 7..10: tile radix passes
-  kStageProjectBwd = 11,
   kStageExpand = 12,  // chunk counter of the duplication expansion
   kStageCount = 13
 };
@@ -183,8 +187,8 @@ struct s3r_workspace {
   uint2* row_spans;         // [rows_cap] column interval of one rectangle row, and the splat's tiles before it
   int64_t rows_cap;
   uint32_t* dup_chunk;      // [K/kDupChunkMin + 2] sorted splat holding the first pair of each expansion chunk
-  uint32_t* contrib;        // [4][K/32 + 2] bit per (warp block, sorted pair): blended in the forward
-  int64_t contrib_words;    // words per warp block
+  uint32_t* contrib;        // [kBlendBands][K/32 + 2] bit per (band, sorted pair): blended in the forward
+  int64_t contrib_words;    // words per band
   int64_t bytes;
   // host-side state of the current call sequence
   s3r::ViewSet views;
