@@ -74,9 +74,9 @@ void free_all(s3r_workspace* ws) {
   void* ptrs[] = {ws->ctr, ws->hist, ws->lookback, ws->selected, ws->frustum_mask,
                   ws->keep_mask, ws->splat_start, ws->kept_list, ws->kept_bits, ws->sp_rgb_d,
                   ws->sp_rect, ws->sp_view, ws->sp_tin, ws->depth_key[0], ws->depth_key[1],
-                  ws->depth_val[0], ws->depth_val[1], ws->dup_key[0], ws->dup_key[1],
-                  ws->dup_val[0], ws->dup_val[1], ws->ranges, ws->final_T, ws->n_contrib,
-                  ws->sp_grad, ws->pose_dM, ws->world_acc, ws->mats, ws->dup_excl, ws->dup_meta, ws->sp_tiles, ws->sp_region, ws->row_spans, ws->dup_chunk, ws->tile_class_cnt, ws->tile_class_list, ws->contrib};
+                  ws->depth_val[0], ws->depth_val[1], ws->dup_key[0], ws->dup_val[0],
+                  ws->pair_scratch, ws->ranges, ws->final_T, ws->n_contrib,
+                  ws->sp_grad, ws->pose_dM, ws->world_acc, ws->mats, ws->dup_excl, ws->dup_meta, ws->sp_tiles, ws->sp_region, ws->dup_chunk, ws->tile_class_cnt, ws->tile_class_list, ws->contrib};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -199,9 +199,7 @@ s3r_status s3r_workspace_create(const s3r_capacity* cap, int device, s3r_workspa
   S3R_ALLOC(ws->depth_val[0], S);
   S3R_ALLOC(ws->depth_val[1], S);
   S3R_ALLOC(ws->dup_key[0], K);
-  S3R_ALLOC(ws->dup_key[1], K);
   S3R_ALLOC(ws->dup_val[0], K);
-  S3R_ALLOC(ws->dup_val[1], K);
   S3R_ALLOC(ws->ranges, cap->max_tiles);
   S3R_ALLOC(ws->tile_class_cnt, 64);
   S3R_ALLOC(ws->tile_class_list, (int64_t)kTileClasses * cap->max_tiles);
@@ -217,7 +215,11 @@ s3r_status s3r_workspace_create(const s3r_capacity* cap, int device, s3r_workspa
   S3R_ALLOC(ws->sp_region, 8 * S);
   // about 2.5 rows per splat at 1 px LOD; past the table, rows are recomputed
   ws->rows_cap = std::min<int64_t>(cap->max_rows > 0 ? cap->max_rows : 4 * S, 0xfffffff0LL);
-  S3R_ALLOC(ws->row_spans, ws->rows_cap);
+  const int64_t pair_words = (K + 63) / 64 * 64;   // the second buffer's start stays aligned
+  S3R_ALLOC(ws->pair_scratch, std::max<int64_t>(2 * pair_words, 2 * ws->rows_cap));
+  ws->dup_key[1] = ws->pair_scratch;
+  ws->dup_val[1] = ws->pair_scratch + pair_words;
+  ws->row_spans = reinterpret_cast<uint2*>(ws->pair_scratch);
   S3R_ALLOC(ws->dup_chunk, K / kDupChunkMin + 2);
   ws->contrib_words = K / 32 + 2;
   S3R_ALLOC(ws->contrib, kBlendBands * ws->contrib_words);

@@ -168,8 +168,10 @@ struct s3r_workspace {
   uint32_t* sp_tin;         // [S] x 8: position, conic, opacity and tile extent (one 32-byte record)
   uint32_t* depth_key[2];   // [S]
   uint32_t* depth_val[2];   // [S]
-  uint32_t* dup_key[2];     // [K]
-  uint32_t* dup_val[2];     // [K]
+  uint32_t* dup_key[2];     // [K], the second in pair_scratch
+  uint32_t* dup_val[2];     // [K], the second in pair_scratch
+  uint32_t* pair_scratch;   // the row table until the pairs are expanded, then the pairs' second
+                            // buffers, which the tile passes write for the first time
   uint2* ranges;            // [tiles]
   uint32_t* tile_class_cnt; // [64] tiles per class of pair count (kTileClasses used)
   uint32_t* tile_class_list;  // [kTileClasses][max_tiles] tile ids per class
@@ -185,6 +187,7 @@ struct s3r_workspace {
   uint32_t* sp_tiles;       // [S] tiles of its rectangle a splat's alpha region reaches, depth order
   float* sp_region;         // [S] x 8: that region, where the row table had no room
   uint2* row_spans;         // [rows_cap] column interval of one rectangle row, and the splat's tiles before it
+                            // (in pair_scratch)
   int64_t rows_cap;
   uint32_t* dup_chunk;      // [K/kDupChunkMin + 2] sorted splat holding the first pair of each expansion chunk
   uint32_t* contrib;        // [kBlendBands][K/32 + 2] bit per (band, sorted pair): blended in the forward

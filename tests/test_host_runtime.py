@@ -74,3 +74,24 @@ def test_one_thread_steps_on_two_devices(lib, degree, n_inst):
         assert lib.fake_launches(device, b"13k_project_bwdI") == before + 1
     for ws in spaces:
         lib.s3r_workspace_destroy(ws)
+
+
+# small image, 1080p view, seven-camera rig, and a row table larger than the pairs
+@pytest.mark.parametrize("cap,most", [
+    (dict(max_gaussians=22_000, max_splats=22_000, max_duplicates=1 << 21, max_views=1, max_instances=2,
+          max_tiles=240, max_pixels=61_440), 41_404_064),
+    (dict(max_gaussians=1_100_000, max_splats=1_100_000, max_duplicates=8_800_000, max_views=1, max_instances=20,
+          max_tiles=8160, max_pixels=2_073_600), 424_125_164),
+    (dict(max_gaussians=9_000_000, max_splats=18_000_000, max_duplicates=144_000_000, max_views=7, max_instances=80,
+          max_tiles=57_600, max_pixels=13_000_000), 6_544_673_372),
+    (dict(max_gaussians=300_000, max_splats=300_000, max_duplicates=3_000_000, max_views=2, max_instances=0,
+          max_tiles=4000, max_pixels=1_000_000, max_rows=3_000_000), 136_828_636)], ids=["tiny", "mid", "rig", "rows"])
+def test_workspaces_stay_within_what_four_byte_rows_took(lib, cap, most):
+    """A workspace takes no more device memory than with the row table of four
+    bytes a row, and s3r_workspace_bytes is what was allocated."""
+    before = lib.fake_allocated()
+    ws = _workspace(lib, **cap)
+    taken = lib.s3r_workspace_bytes(ws)
+    assert taken == lib.fake_allocated() - before
+    assert taken <= most
+    lib.s3r_workspace_destroy(ws)
