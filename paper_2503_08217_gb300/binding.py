@@ -176,11 +176,17 @@ def _ptr(t) -> int | None:
     return t.data_ptr()
 
 
+# The current stream's raw handle: a torch.cuda.current_stream() object took 8 us per
+# call. Not a public function, so the object serves where a torch has none.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None) -> int:
     if stream is not None:
         return stream.cuda_stream
-    # the raw handle: a torch.cuda.current_stream() object took 8 us per call
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def make_camera(cam) -> Camera:

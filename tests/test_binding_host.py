@@ -37,3 +37,13 @@ def test_camera_matrix_takes_what_float_takes(w):
 def test_camera_matrix_refuses_the_rest(w):
     with pytest.raises((TypeError, ValueError)):
         _camera(w)
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_current_stream_with_and_without_the_raw_handle(monkeypatch, raw):
+    import torch
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x77))
+    monkeypatch.setattr(binding, "_raw_stream", (lambda device: 0x70 + device) if raw else None)
+    assert binding._stream() == (0x73 if raw else 0x77)
+    assert binding._stream(types.SimpleNamespace(cuda_stream=5)) == 5
