@@ -23,6 +23,8 @@
 // adjoints (uv, conic, opacity, rgb) are summed over the warp through shared
 // memory, then over the CTA (one shared atomic per two splats and warp),
 // and flushed to global memory with one vector atomic per four floats.
+#include <type_traits>
+
 #include "s3r_internal.cuh"
 
 namespace s3r {
@@ -391,7 +393,10 @@ __device__ __forceinline__ float4 alpha_box(const float2 xy, const float4 co) {
   const float o = co.w;
   if (!(o * 255.f > 1.f)) return make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
   const float det = conic_det_lower(co.x, co.y, co.z);
-  if (det < 0.f) return make_float4(-INFINITY, INFINITY, -INFINITY, INFINITY);
+  if (det < 0.f) {
+    const float sum = co.x + co.y + co.z;
+    return make_float4(sum != sum ? sum : -INFINITY, INFINITY, -INFINITY, INFINITY);
+  }
   const float L2 = 2.f * __logf(255.f * o);
   const float ex = sqrtf(fmaxf(L2 * co.z / det, 0.f)) * 1.002f + 0.02f;
   const float ey = sqrtf(fmaxf(L2 * co.x / det, 0.f)) * 1.002f + 0.02f;
@@ -512,7 +517,7 @@ __device__ __forceinline__ float blend_alpha(float p, float al, float nT, int po
 // definition never reaches the cap for those splats either.
 //
 // fwd_eval: the exponents and alphas, which depend on the splat and the pixel
-// alone. `cap`: the alpha cap, or infinity where the splat cannot reach it.
+// alone. `cap`: the alpha cap, or NaN where the splat cannot reach it.
 // fwd_apply: the decisions and the compositing, in the splats' order.
 template <int kPairs>
 struct SplatEval {
@@ -573,6 +578,16 @@ __device__ __forceinline__ void fwd_apply(const SplatEval<kPairs>& e, const floa
   float s0, s1;
   upk(ab_sum, s0, s1);
   any_blend = s0 + s1 > 0.f;
+}
+
+// A splat without a conic (an entry NaN: a Gaussian so long that its 2D covariance
+// overflows) has alpha NaN, and makes NaN of the pixels that walk it. The decisions
+// let NaN pass, as those of a splat that a pixel takes, so a pixel that has stopped
+// is given alpha 0 here.
+template <int kPairs>
+__device__ __forceinline__ void guard_stopped(SplatEval<kPairs>& e, const float (&floor_)[2 * kPairs]) {
+#pragma unroll
+  for (int k = 0; k < 2 * kPairs; ++k) e.al[k] = floor_[k] > 1.f ? 0.f : e.al[k];
 }
 
 template <int kPix>
@@ -695,66 +710,79 @@ __global__ void __launch_bounds__(32 * kWarpsT, S3R_BLEND_FWD_BLOCKS * kBandWarp
         if (__all_sync(0xffffffffu, all_stopped(floor_))) break;
         // which of the next 32 splats can reach alpha >= 1/255 in this warp's band
         const int jl = c0 + (int)lane;
-        bool reach = false;
+        bool reach = false, no_conic = false;
         if (jl < m) {
           const float4 p0 = s_p0[jl], p1 = s_p1[jl], p3 = s_p3[jl];
           const float4 ea = make_float4(s_u[jl].x, p3.z, p0.x, p0.z);
           const float4 eb = make_float4(p1.x, p1.z, 0.f, 0.f);
-          reach = !box_misses(s_box[jl], P) && ellipse_reaches(ea, eb, P);
+          const float4 box = s_box[jl];
+          reach = !box_misses(box, P) && ellipse_reaches(ea, eb, P);
+          no_conic = box.x != box.x;
         }
         uint32_t todo = __ballot_sync(0xffffffffu, reach);
         uint32_t blended = 0;     // splats of this chunk blended into some pixel of the band
-        if constexpr (kWarpsT == 2) {
-          while (todo) {
-            const int j = c0 + __ffs(todo) - 1;
-            todo &= todo - 1;
-            const float4 q0 = s_p0[j], q1 = s_p1[j], q2 = s_p2[j], q3 = s_p3[j];
-            const float2 qu = s_u[j];
-            bool any_blend = false;
-            SplatEval<kPairs> e;
-            // warp-uniform: every lane walks the same splat
-            if (q1.z > kAlphaMax) {
-              fwd_eval<true, kPairs>(q0, q1, q3, qu, kAlphaMax, FY, FX, e);
-              fwd_apply<kCount, kPairs>(e, q2, q3, ONE, b0 + j + 1, T2, C2, last, endp, floor_, n_eval,
-                                        any_blend);
-            } else {
-              fwd_eval<false, kPairs>(q0, q1, q3, qu, 0.f, FY, FX, e);
-              fwd_apply<kCount, kPairs>(e, q2, q3, ONE, b0 + j + 1, T2, C2, last, endp, floor_, n_eval,
-                                        any_blend);
-            }
-            if (__any_sync(0xffffffffu, any_blend)) blended |= 1u << (j - c0);
-          }
-        } else {
-          // kAhead splats at a time: their exponents and alphas are independent
-          // and overlap, only the compositing is a chain
-          while (todo) {
-            int js[kAhead];
-            SplatEval<kPairs> e[kAhead];
-            int m_here = 0;
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-              js[u] = c0 + (todo ? __ffs(todo) - 1 : 0);
-              m_here += todo ? 1 : 0;
+        // the chunk's walk; kGuard where it has a splat without a conic (see guard_stopped)
+        auto walk = [&](auto guard) {
+          constexpr bool kGuard = decltype(guard)::value;
+          if constexpr (kWarpsT == 2) {
+            while (todo) {
+              const int j = c0 + __ffs(todo) - 1;
               todo &= todo - 1;
-            }
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-              const int j = js[u];
-              const float4 q1 = s_p1[j];
-              fwd_eval<true, kPairs>(s_p0[j], q1, s_p3[j], s_u[j], q1.z > kAlphaMax ? kAlphaMax : INFINITY,
-                                     FY, FX, e[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-              if (u >= m_here) break;
-              const int j = js[u];
+              const float4 q0 = s_p0[j], q1 = s_p1[j], q2 = s_p2[j], q3 = s_p3[j];
+              const float2 qu = s_u[j];
               bool any_blend = false;
-              fwd_apply<kCount, kPairs>(e[u], s_p2[j], s_p3[j], ONE, b0 + j + 1, T2, C2, last, endp, floor_,
-                                        n_eval, any_blend);
+              SplatEval<kPairs> e;
+              // warp-uniform: every lane walks the same splat
+              if (q1.z > kAlphaMax) {
+                fwd_eval<true, kPairs>(q0, q1, q3, qu, kAlphaMax, FY, FX, e);
+                fwd_apply<kCount, kPairs>(e, q2, q3, ONE, b0 + j + 1, T2, C2, last, endp, floor_, n_eval,
+                                          any_blend);
+              } else {
+                fwd_eval<false, kPairs>(q0, q1, q3, qu, 0.f, FY, FX, e);
+                if constexpr (kGuard) guard_stopped<kPairs>(e, floor_);
+                fwd_apply<kCount, kPairs>(e, q2, q3, ONE, b0 + j + 1, T2, C2, last, endp, floor_, n_eval,
+                                          any_blend);
+              }
               if (__any_sync(0xffffffffu, any_blend)) blended |= 1u << (j - c0);
             }
+          } else {
+            // kAhead splats at a time: their exponents and alphas are independent
+            // and overlap, only the compositing is a chain
+            while (todo) {
+              int js[kAhead];
+              SplatEval<kPairs> e[kAhead];
+              int m_here = 0;
+#pragma unroll
+              for (int u = 0; u < kAhead; ++u) {
+                js[u] = c0 + (todo ? __ffs(todo) - 1 : 0);
+                m_here += todo ? 1 : 0;
+                todo &= todo - 1;
+              }
+#pragma unroll
+              for (int u = 0; u < kAhead; ++u) {
+                const int j = js[u];
+                const float4 q1 = s_p1[j];
+                // where there is no cap, NaN: the minimum is then the alpha, NaN included
+                fwd_eval<true, kPairs>(s_p0[j], q1, s_p3[j], s_u[j], q1.z > kAlphaMax ? kAlphaMax : NAN, FY, FX,
+                                       e[u]);
+              }
+#pragma unroll
+              for (int u = 0; u < kAhead; ++u) {
+                if (u >= m_here) break;
+                const int j = js[u];
+                bool any_blend = false;
+                if constexpr (kGuard) guard_stopped<kPairs>(e[u], floor_);
+                fwd_apply<kCount, kPairs>(e[u], s_p2[j], s_p3[j], ONE, b0 + j + 1, T2, C2, last, endp, floor_,
+                                          n_eval, any_blend);
+                if (__any_sync(0xffffffffu, any_blend)) blended |= 1u << (j - c0);
+              }
+            }
           }
-        }
+        };
+        if (__ballot_sync(0xffffffffu, no_conic))
+          walk(std::true_type{});
+        else
+          walk(std::false_type{});
         if (lane == 0 && blended) or_bits(wbits, range.x + b0 + c0, blended);
       }
     }
