@@ -212,3 +212,30 @@ def test_world_adjoints_of_tiny_instances(n_inst):
         assert np.abs(got[0]["inst_quat"][sizes > 0]).max(axis=1).min() > 0
     for k in got[0]:
         np.testing.assert_array_equal(got[0][k], got[1][k])
+
+
+@pytest.mark.parametrize("K,D,S", [(1, 1, 1), (3, 16, 2), (70, 8, 1)])
+def test_ode_trajectory_without_steps(K, D, S):
+    """One output time: the poses are the initial states' own, only they get a
+    gradient, and every other gradient stays exactly what it was."""
+    from paper_2503_08217_gb300 import binding
+    from oracle import ode
+    cu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()   # noqa: E731
+    params, embed, z0 = scenegen.ode_model(79, K, D)
+    rng = np.random.default_rng(83)
+    times = np.array([0.3], np.float32)
+    p, e, z, t = cu(params), cu(embed), cu(z0), cu(times)
+    states, quat, trans = binding.ode_poses(p, e, z, t, S)
+    np.testing.assert_array_equal(states.cpu().numpy().reshape(-1), z0.reshape(-1))
+    np.testing.assert_array_equal(trans.cpu().numpy().reshape(K, 3), z0[:, :3])
+    gq, gt = rng.standard_normal((1, K, 4)).astype(np.float32), rng.standard_normal((1, K, 3)).astype(np.float32)
+    g_params, g_embed = torch.full((params.size,), 0.5, device="cuda"), torch.full((K, D), -0.25, device="cuda")
+    g_z0 = torch.zeros((K, 6), device="cuda")
+    gq_t, gt_t = cu(gq), cu(gt)
+    binding.ode_poses_bwd(p, e, t, S, states, gq_t, gt_t, g_params, g_embed, g_z0)
+    torch.cuda.synchronize()
+    assert (g_params == 0.5).all() and (g_embed == -0.25).all()
+    want = ode.backward(params, embed, z0, times, S, 64, gq.astype(np.float64), gt.astype(np.float64))[2]
+    a = g_z0.double().cpu().numpy()
+    np.testing.assert_array_equal(a[:, :3], gt[0])
+    assert np.linalg.norm(a - want) <= 1e-5 * np.linalg.norm(want)
