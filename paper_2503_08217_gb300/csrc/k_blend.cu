@@ -57,7 +57,8 @@ constexpr float kTStop = 1e-4f;
 // longest, 32 the empty tiles). Chunks of memory-bound zeroing are spread
 // evenly between the tiles (position i is a chunk when floor((i+1) C / P)
 // > floor(i C / P), C chunks among P positions), so that their stores run
-// while other CTAs of the SM blend: the forward clears the per-splat adjoints
+// while other CTAs of the SM blend (where the forward has a CTA for every tile they
+// follow the tiles instead): the forward clears the per-splat adjoints
 // the backward sums into, the backward in overwrite mode clears the caller's
 // gradient arrays. The last CTA to leave resets the cursor for the next launch.
 struct TileQueue {
@@ -183,9 +184,9 @@ __device__ __forceinline__ void queue_exit(const TileQueue& q) {
 // with one compare per lane. A CTA's first position is its own number, the cursor
 // counts those after the grid: an SM's CTAs start together, and where they drew
 // their first positions from the cursor, the longest lists met on one SM. Where
-// the launch has a CTA for every tile it is direct: CTA i takes tile i, then the zeroing chunks grid - 1 - i, + grid, ...,
-// so that the chunks go to the CTAs without a tile or with the shortest ones
-// first and the cursor stays untouched. (Chunks spread among the tiles, as the
+// the launch has a CTA for every tile it is direct: CTA i takes tile i, then the
+// zeroing chunks grid - 1 - i, + grid, ..., so that the chunks go to the CTAs
+// without a tile or with the shortest ones first and the cursor stays untouched. (Chunks spread among the tiles, as the
 // cursor hands them out, held the last tiles back until others had ended: 1,196
 // tiles of a view of 381,000 splats 86 us, 57 us without any zeroing.)
 struct QueueState {
@@ -492,7 +493,8 @@ constexpr int kBatchFwd = S3R_BLEND_FWD_BATCH;
 // `floor_` is the least alpha the pixel still takes: 1/255 until it stops, then
 // infinity. The splat is taken where p <= 0, alpha >= floor_ and the
 // transmittance nT it would leave is not under 1e-4; where only the last fails
-// the pixel stops. It took 6.5 % off the kernel's instructions. Returns the applied alpha and moves the last position.
+// the pixel stops. It took 6.5 % off the kernel's instructions. Returns the
+// applied alpha and moves the last position.
 __device__ __forceinline__ float blend_alpha(float p, float al, float nT, int pos, float& floor_,
                                              int& last) {
   float ab;
@@ -510,8 +512,8 @@ __device__ __forceinline__ float blend_alpha(float p, float al, float nT, int po
 
 // One splat of the forward's walk over a lane's pixels, kPairs packed pairs:
 // two columns of two rows each with two warps per tile, one row of two columns
-// with four (FX and FY hold the pairs' pixel centres accordingly). kClamp: the splat's opacity exceeds 0.99, so alpha = o G may
-// reach the 0.99 cap; for o <= 0.99 it cannot (G = 2^p <= 1 where p <= 0, up
+// with four (FX and FY hold the pairs' pixel centres accordingly). kClamp: the
+// splat's opacity exceeds 0.99, so alpha = o G may reach the 0.99 cap; for o <= 0.99 it cannot (G = 2^p <= 1 where p <= 0, up
 // to the last ulp of ex2.approx at p = 0), and the clamp is left out. The
 // backward takes the same branch per splat, and the FP64 o G of the exact
 // definition never reaches the cap for those splats either.

@@ -315,7 +315,7 @@ constexpr int kExpItems = S3R_DUP_EXPAND_ITEMS;       // outputs per thread per 
 constexpr int kExpChunk = kDupThreads * kExpItems;    // outputs per chunk
 static_assert(kExpChunk >= kDupChunkMin, "the chunk map is sized for chunks of kDupChunkMin");
 static_assert(kExpChunk % 32 == 0, "a chunk clears whole words of contributor bits");
-static_assert(kExpItems <= 14, "above 14 outputs per thread the larger chunks measured slower");
+static_assert(kExpItems <= 14, "not built above 14 outputs per thread (16 took 0.148 ms where 12 took 0.137)");
 
 constexpr float kSpanPad = 0.05f;        // pixels, on the strips and the column bounds
 

@@ -497,8 +497,10 @@ __device__ __forceinline__ float approx_rcp(float x) {
 
 // Two FP32 values in one 64-bit register for the packed .f32x2 instructions
 // (sm_100 and later): one instruction does the same IEEE operation on both
-// halves, so pairs cost half the issue slots of scalar code with bit-identical
-// results.
+// halves, with bit-identical results. It takes the issue cycles of two scalar ones
+// (an FMA 2.1 measured, a scalar one 1.03), so that what pairs save is instructions
+// to fetch and schedule, not arithmetic time: with scalar FMAs the blends of the
+// surround rig took 1.284 ms forward and 1.987 backward, against 1.042 and 1.852.
 typedef unsigned long long f2;
 __device__ __forceinline__ f2 pk(float a, float b) {
   f2 r;
