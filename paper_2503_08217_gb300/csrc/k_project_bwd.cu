@@ -65,13 +65,13 @@ constexpr int kPoseCopies = 256;
 // Instance blockIdx.x + 1: its matrix adjoints summed over the copies (which are
 // cleared for the next call; they start at zero with the workspace), then
 // dL/dP_k = V_rot^T dL/dW_{v,k} summed over views, then (q, t) of the pose.
-constexpr int kPoseThreads = 128;
+constexpr int kPoseThreads = 256;
 __global__ void __launch_bounds__(kPoseThreads) k_pose_chain(const __grid_constant__ ViewSet vs, float* dM,
                                                              int n_inst,
                                                              const float4* pose_q, float* g_q, float* g_t,
                                                              int overwrite) {
   sequence_begin();
-  constexpr int kParts = 8;   // threads that share a sum, every eighth copy each
+  constexpr int kParts = 16;   // threads that share a sum, every sixteenth copy each
   static_assert(kPoseCopies % kParts == 0, "as many copies for each part");
   __shared__ float s_part[S3R_MAX_VIEWS * 12][kParts + 1];
   __shared__ float s_d[S3R_MAX_VIEWS][12];
