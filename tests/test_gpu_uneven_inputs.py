@@ -239,3 +239,42 @@ def test_ode_trajectory_without_steps(K, D, S):
     a = g_z0.double().cpu().numpy()
     np.testing.assert_array_equal(a[:, :3], gt[0])
     assert np.linalg.norm(a - want) <= 1e-5 * np.linalg.norm(want)
+
+
+def test_captured_forward_chooses_at_replay():
+    """A forward captured on evenly filled tiles and replayed on splats massed in a
+    few (and back) renders what a call does: which launch works is decided on the
+    device. The images have tile counts at which the lists choose."""
+    import gpu_helpers
+    from paper_2503_08217_gb300.render import DeviceScene
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = 14 * sms // 40                                   # 40 x rows tiles, between 9 and 18 per SM
+    count = 20_000
+    rng = np.random.default_rng(89)
+    g = scenegen.generate("fd", seed=9, n_static=count, n_inst=0, n_steps=2)
+    cam = make_camera(640, 16 * rows, 320.0, (0.0, 0.0, 0.0), 0.0)
+    g = scenegen.with_cameras(g, [[cam], [cam]])
+    g.log_scales[:] = np.log(rng.uniform(0.005, 0.03, (count, 3)))
+    z = rng.uniform(4, 12, count)
+    xy = rng.uniform(-1, 1, (count, 2)) * z[:, None]
+    places = [np.concatenate([e * xy, z[:, None]], 1).astype(np.float32) for e in (0.95, 0.02)]
+    g.means[:] = places[0]
+    dev = DeviceScene.from_host(g)
+    vis = torch.from_numpy(oracle.vis_reset(count)[0]).cuda()
+    bg = torch.tensor([0.2, 0.4, 0.6], device="cuda")
+    iq = torch.from_numpy(np.ascontiguousarray(g.inst_quat[0], np.float32)).cuda()
+    it = torch.from_numpy(np.ascontiguousarray(g.inst_trans[0], np.float32)).cuda()
+    make = lambda: gpu_helpers.Renderer(count, 0, [cam], max_duplicates=1 << 20)      # noqa: E731
+    r, eager = make(), make()
+    out = torch.empty(3 * cam.width * cam.height, device="cuda")
+    graph = r.capture(lambda: r.forward(dev, iq, it, [cam], 0.0, vis, None, 0.0, bg, out))
+    for place in (0, 1, 0, 1):
+        dev.means.copy_(torch.from_numpy(places[place]).cuda())
+        out.fill_(float("nan"))
+        graph.replay()
+        want = eager.forward(dev, iq, it, [cam], 0.0, vis, None, 0.0, bg)
+        torch.cuda.synchronize()
+        ranges = r.ws.debug("tile_ranges", torch.int32, 80 * rows).view(-1, 2)
+        longest, pairs = int((ranges[:, 1] - ranges[:, 0]).max()), r.counts()["n_duplicates"]
+        assert (longest * 40 * rows > 6 * pairs) == (place == 1) and pairs < 300_000
+        np.testing.assert_array_equal(out.cpu().numpy(), want.cpu().numpy())
