@@ -72,9 +72,8 @@ __global__ void __launch_bounds__(kPoseThreads) k_pose_chain(const __grid_consta
                                                              int overwrite) {
   sequence_begin();
   constexpr int kParts = 16;   // threads that share a sum, every sixteenth copy each
-  static_assert(kPoseCopies % kParts == 0 && kPoseCopies / kParts <= 16, "as many copies for each part, a bit each");
+  static_assert(kPoseCopies % kParts == 0, "as many copies for each part");
   __shared__ float s_part[S3R_MAX_VIEWS * 12][kParts + 1];
-  __shared__ uint16_t s_used[S3R_MAX_VIEWS * 12 * kParts];   // copies with anything to clear
   __shared__ float s_d[S3R_MAX_VIEWS][12];
   __shared__ float s_P[12];
   const int nk = n_inst + 1, k = (int)blockIdx.x + 1;
@@ -87,23 +86,14 @@ __global__ void __launch_bounds__(kPoseThreads) k_pose_chain(const __grid_consta
 #pragma unroll
     for (int c = 0; c < kPoseCopies / kParts; ++c) x[c] = p[(c * kParts + part) * stride];
     float sum = 0.f;
-    uint32_t used = 0;
 #pragma unroll
     for (int c = 0; c < kPoseCopies / kParts; ++c) {
       sum += x[c];
-      used |= x[c] != 0.f ? 1u << c : 0u;
+      if (x[c] != 0.f) p[(c * kParts + part) * stride] = 0.f;
     }
     s_part[i][part] = sum;
-    s_used[j] = (uint16_t)used;
   }
   __syncthreads();
-  // cleared once every thread has its sums: loads after stores waited for them
-  for (int j = threadIdx.x; j < sums * kParts; j += kPoseThreads) {
-    const int part = j / sums, i = j - part * sums, v = i / 12, e = i - 12 * v;
-    float* p = dM + (v * nk + k) * 12 + e;
-    for (uint32_t used = s_used[j]; used; used &= used - 1)
-      p[((__ffs(used) - 1) * kParts + part) * stride] = 0.f;
-  }
   for (int i = threadIdx.x; i < sums; i += kPoseThreads) {
     float sum = 0.f;
 #pragma unroll
